@@ -97,8 +97,9 @@ def cod_select(n: int, K: int, r: float, r_min: float, seed: int, sample_id: int
     """COD data construction for one sample (pard_cod_select): returns device
     tensors keep [K-1, n] and counts [K] (int32), enqueued on `stream`."""
     import torch
-    keep = torch.zeros((max(K - 1, 1), n), dtype=torch.int32, device="cuda")
-    counts = torch.zeros(K, dtype=torch.int32, device="cuda")
+    # the kernel writes every flag and count
+    keep = torch.empty((max(K - 1, 1), n), dtype=torch.int32, device="cuda")
+    counts = torch.empty(K, dtype=torch.int32, device="cuda")
     s = stream if stream is not None else torch.cuda.current_stream()
     _check(lib().pard_cod_select(n, K, float(r), float(r_min), seed, sample_id, keep.data_ptr(), counts.data_ptr(),
                                  s.cuda_stream), "pard_cod_select")

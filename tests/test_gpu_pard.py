@@ -471,3 +471,19 @@ def test_state_errors_are_reported():
     with pytest.raises(pard.PardError) as e:
         P.eng.prefill([list(range(10))], 10_000, wl.K)
     assert e.value.code == -1
+
+
+def test_cod_threshold_bins_at_the_edges():
+    """COD rows at the edges of the four-rows-a-thread split and of the
+    threshold search: row counts around multiples of four, keep counts of
+    zero, of one and of every candidate, and more subtasks than rows."""
+    import torch
+    from oracle import cod
+    from paper_2504_18583_gb300 import pard
+    for t, (n, K, r, r_min) in enumerate([(3, 6, 0.9, 0.0), (5, 4, 0.01, 0.0), (127, 12, 0.95, 0.0), (4093, 3, 0.999, 0.0),
+                                          (4095, 16, 0.5, 0.001), (4096, 3, 1.0, 0.0), (8, 64, 1.0, 1.0)]):
+        keep_g, counts_g = pard.cod_select(n, K, r, r_min, seed=(1 << 40) + t, sample_id=7 * t)
+        keep_o, counts_o = cod.cod_select(n, K, r, r_min, seed=(1 << 40) + t, sample_id=7 * t)
+        torch.cuda.synchronize()
+        assert counts_g.cpu().tolist() == counts_o, (n, K, r, r_min)
+        assert np.array_equal(keep_g.cpu().numpy(), keep_o), (n, K, r, r_min)
