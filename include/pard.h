@@ -262,7 +262,7 @@ pard_status pard_unpack_weights(pard_ctx* ctx, void* stream);
  * after the emitted tokens).  A candidate outside [0, vocab) is never read
  * from the logits: it counts as a rejection at its offset.  Nothing is
  * committed anywhere: no context is involved.
- * Scratch: one fixed file-scope device array of about 6.3 MiB, sized for
+ * Scratch: one fixed file-scope device array of about 340 KiB, sized for
  * batch <= 16, 1 <= K <= 8, vocab <= 128256 (vocab a multiple of 8); larger
  * sizes return PARD_ERR_ARG with a message.  Every GPU that loads the
  * library keeps that array until the process exits.  The first call on a

@@ -197,6 +197,26 @@ struct AcceptArgs {
   int* kv_slots;
   int* n_emit;
   uint32_t* status;        // sticky device status word (null: none)
+  const float4* dstats;    // sampling: tile statistics of the draft rows b K + i (null: their normalisers are in st.dnorm)
+  int d_m_cap;
+};
+
+// Statistics of given logits in tiles of kGivenTile entries, for the
+// acceptance that keeps its scratch in a fixed array (noalloc.cu).
+constexpr int kGivenTile = 2048;
+struct GivenArgs {
+  const float* y;          // [rows_t][vocab]
+  const float* z;          // [rows_d][vocab] (rows_d = 0: none)
+  int rows_t, rows_d, m_cap_t, m_cap_d, vocab;
+  int vec;                 // both arrays are 16-byte aligned
+  int sample;
+  float4 *stats_t, *stats_d;
+  int2* stats_it;
+  CallArgs call;           // written to *call_out with the reset state below
+  CallArgs* call_out;
+  DevState st;
+  const int* d;            // [batch][K] candidates
+  int batch, K;
 };
 
 constexpr int kMaxGemmTiles = 32768;  // output tiles (weight tile x token tile) of one GEMM launch
@@ -210,6 +230,7 @@ void launch_gather_rows(const __nv_bfloat16* x, int x_rows, const float* ssq, in
                         bool pdl);
 void launch_pack(const __nv_bfloat16* tmp, __nv_bfloat16* w, int R, int K, int nblocks, bool unpack, cudaStream_t s);
 void launch_select(const SelectArgs& a, cudaStream_t s, bool pdl);
+void launch_given_stats(const GivenArgs& a, cudaStream_t s);
 void launch_accept_greedy(const AcceptArgs& a, cudaStream_t s, bool pdl);
 void launch_accept_sample(const AcceptArgs& a, cudaStream_t s, bool pdl);
 void launch_row_stats(const float* logits, int rows, int vocab, int w_tiles, int m_cap, const CallArgs* call,

@@ -254,6 +254,56 @@ __device__ RowRed reduce_row(const float4* stats, const int2* stats_i, int w_til
   return out;
 }
 
+// The same for rows m0 .. m0 + nrows - 1 at once (nrows <= 32), by a block of
+// 32 warps: 32 / nrows warps share a row, each lane takes every 32nd of its
+// warp's tiles and the warp merges by shuffles, then one thread a row merges
+// the warps in order.  out[i] holds row i when the call returns.  (One row
+// after the other through a block-wide tree cost about 2.5 us a row.)
+constexpr int kRowWarps = 32;
+template <bool kLse>
+__device__ void reduce_rows(const float4* stats, const int2* stats_i, int w_tiles, int m_cap, int m0, int nrows,
+                            float T, RowRed* part, RowRed* out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int per = kRowWarps / nrows;  // warps a row
+  if (warp < per * nrows) {
+    const int m = m0 + warp / per;
+    RowRed r{-INFINITY, INT_MAX, 0.f, -INFINITY, INT_MAX};
+#pragma unroll 4
+    for (int t = (warp % per) * 32 + lane; t < w_tiles; t += 32 * per) {
+      const size_t at = (size_t)t * m_cap + m;
+      if constexpr (kLse) {
+        const float4 s = stats[at];
+        merge_lse(r.mx, r.se, s.x, s.y, T);
+      } else {
+        argmax_merge(r.mx, r.arg, stats[at].x, stats_i[at].x);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, r.mx, o);
+      if constexpr (kLse) {
+        const float s2 = __shfl_xor_sync(0xffffffffu, r.se, o);
+        merge_lse(r.mx, r.se, m2, s2, T);
+      } else {
+        const int a2 = __shfl_xor_sync(0xffffffffu, r.arg, o);
+        argmax_merge(r.mx, r.arg, m2, a2);
+      }
+    }
+    if (lane == 0) part[warp] = r;
+  }
+  __syncthreads();
+  if ((int)threadIdx.x < nrows) {
+    RowRed r = part[threadIdx.x * per];
+    for (int i = 1; i < per; ++i) {
+      const RowRed o = part[threadIdx.x * per + i];
+      if constexpr (kLse) merge_lse(r.mx, r.se, o.mx, o.se, T);
+      else argmax_merge(r.mx, r.arg, o.mx, o.arg);
+    }
+    out[threadIdx.x] = r;
+  }
+  __syncthreads();
+}
+
 // Draft tokens (argmax or Gumbel-max winner) and draft-row normalisers;
 // or the prefill's first token and state initialisation.
 __global__ void __launch_bounds__(256) select_kernel(const __grid_constant__ SelectArgs a) {
@@ -339,16 +389,15 @@ __device__ void commit_seq(const AcceptArgs& a, int b, int acc, const int* emitt
 }
 
 // Greedy: a = longest prefix with d_i == argmax y_i, bonus = argmax y_a.
-__global__ void __launch_bounds__(256) accept_greedy_kernel(const __grid_constant__ AcceptArgs a) {
+__global__ void __launch_bounds__(32 * kRowWarps) accept_greedy_kernel(const __grid_constant__ AcceptArgs a) {
   pdl_wait();
   pdl_trigger();
-  __shared__ RowRed sred[256];
+  __shared__ RowRed s_part[kRowWarps], s_row[17];
   __shared__ int s_arg[17];
   const int b = blockIdx.x;
-  for (int i = 0; i <= a.K; ++i) {
-    const RowRed r = reduce_row(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1) + i, 1.0f, sred);
-    if (threadIdx.x == 0) s_arg[i] = r.arg;
-  }
+  reduce_rows<false>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, 1.0f, s_part, s_row);
+  if ((int)threadIdx.x <= a.K) s_arg[threadIdx.x] = s_row[threadIdx.x].arg;
+  __syncthreads();
   if (threadIdx.x != 0) return;
   int acc = 0;
   while (acc < a.K && a.st.d[b * a.st.kmax + acc] == s_arg[acc]) ++acc;
@@ -364,22 +413,26 @@ __global__ void __launch_bounds__(256) accept_greedy_kernel(const __grid_constan
 }
 
 void launch_accept_greedy(const AcceptArgs& a, cudaStream_t s, bool pdl) {
-  PARD_LAUNCH(accept_greedy_kernel, a.batch, 256, 0, s, pdl, a);
+  PARD_LAUNCH(accept_greedy_kernel, a.batch, 32 * kRowWarps, 0, s, pdl, a);
 }
 
 // Sampling, phase 1: row normalisers and the accept tests
 // u_i * q_i(d_i) < p_i(d_i), p = softmax(y/T), q = softmax(z/T).
-__global__ void __launch_bounds__(256) accept_test_kernel(const __grid_constant__ AcceptArgs a) {
+__global__ void __launch_bounds__(32 * kRowWarps) accept_test_kernel(const __grid_constant__ AcceptArgs a) {
   pdl_wait();
   pdl_trigger();
-  __shared__ RowRed sred[256];
-  __shared__ float2 s_norm[17];
+  __shared__ RowRed s_part[kRowWarps], s_row[17], s_drow[16];
+  __shared__ float2 s_norm[17], s_dnorm[16];
   const int b = blockIdx.x;
   const float T = a.call->temp;
-  for (int i = 0; i <= a.K; ++i) {
-    const RowRed r = reduce_row(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1) + i, T, sred);
-    if (threadIdx.x == 0) s_norm[i] = make_float2(r.mx, r.se);
-  }
+  reduce_rows<true>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, T, s_part, s_row);
+  if (a.dstats && a.K > 0)
+    reduce_rows<true>(a.dstats, nullptr, a.w_tiles, a.d_m_cap, b * a.K, a.K, T, s_part, s_drow);
+  if ((int)threadIdx.x <= a.K) s_norm[threadIdx.x] = make_float2(s_row[threadIdx.x].mx, s_row[threadIdx.x].se);
+  if ((int)threadIdx.x < a.K)
+    s_dnorm[threadIdx.x] = a.dstats ? make_float2(s_drow[threadIdx.x].mx, s_drow[threadIdx.x].se)
+                                    : a.st.dnorm[b * a.st.kmax + threadIdx.x];
+  __syncthreads();
   if (threadIdx.x != 0) return;
   int j = a.K;
   for (int i = 0; i < a.K; ++i) {
@@ -392,14 +445,14 @@ __global__ void __launch_bounds__(256) accept_test_kernel(const __grid_constant_
     }
     const float yv = a.logits[((size_t)b * (a.K + 1) + i) * a.vocab + di];
     const float p = expf(yv / T - s_norm[i].x / T) / s_norm[i].y;
-    const float2 zn = a.st.dnorm[b * a.st.kmax + i];
+    const float2 zn = s_dnorm[i];
     const float zv = a.dlogits[((size_t)b * a.K + i) * a.vocab + di];
     const float q = expf(zv / T - zn.x / T) / zn.y;
     const float u = uniform01(philox_word(a.call->seed, STREAM_ACCEPT, a.call->step, (uint32_t)b, (uint32_t)i, 0u));
     if (!(u * q < p)) { j = i; break; }
   }
   a.st.samp_a[b] = j;
-  const float2 zn = j < a.K ? a.st.dnorm[b * a.st.kmax + j] : make_float2(0.f, 1.f);
+  const float2 zn = j < a.K ? s_dnorm[j] : make_float2(0.f, 1.f);
   a.st.samp_norm[b] = make_float4(s_norm[j].x, s_norm[j].y, zn.x, zn.y);
 }
 
@@ -422,18 +475,45 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
   const int v0 = (int)((long)part * a.vocab / kResampleSplit), v1 = (int)((long)(part + 1) * a.vocab / kResampleSplit);
   float best = -INFINITY;
   int bi = INT_MAX;
-  for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
-    const float g = gumbel(philox_word(a.call->seed, STREAM_BONUS, a.call->step, (uint32_t)b, 0u, (uint32_t)v));
-    float sc;
-    if (z) {
-      const float p = expf(y[v] / T - nm.x / T) / nm.y;
-      const float q = expf(z[v] / T - nm.z / T) / nm.w;
-      const float w = fmaxf(p - q, 0.f);
-      sc = w > 0.f ? logf(w) + g : -INFINITY;
-    } else {
-      sc = y[v] / T + g;
+  // A thread takes the four entries of one Philox block at a time.  An entry
+  // whose noise cannot lift it over the warp's best so far is passed over
+  // before the logarithms: its score beats `best` only if -log u < w exp(-best)
+  // (w exp(-best) = exp(y/T - best) without a draft row), and -log u >= 1 - u;
+  // the factor 1.0001 is far above the roundings of both sides.
+  const uint64_t seed = a.call->seed;
+  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32), step = (uint32_t)a.call->step;
+  const float cy = nm.x / T, cz = nm.z / T;
+  for (int blk0 = v0 / 4; 4 * blk0 < v1; blk0 += blockDim.x) {
+    const int blk = blk0 + threadIdx.x;
+    const U4 pw = philox4x32_10(U4{(uint32_t)blk, (uint32_t)STREAM_BONUS << 16, (uint32_t)b, step}, k0, k1);
+    const uint32_t wd[4] = {pw.x, pw.y, pw.z, pw.w};
+    float yv[4], zv[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int v = 4 * blk + e;
+      const bool in = v >= v0 && v < v1;
+      yv[e] = in ? y[v] : 0.f;
+      zv[e] = in && z ? z[v] : 0.f;
     }
-    argmax_merge(best, bi, sc, v);
+    const float wbest = warp_max(best);
+    const float inv_best = expf(-wbest);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int v = 4 * blk + e;
+      if (v < v0 || v >= v1) continue;
+      const float t = 1.0f - uniform_open01(wd[e]);  // exact
+      if (z) {
+        const float p = expf(yv[e] / T - cy) / nm.y;
+        const float q = expf(zv[e] / T - cz) / nm.w;
+        const float w = fmaxf(p - q, 0.f);
+        if (w > 0.f && t > w * inv_best * 1.0001f) continue;
+        argmax_merge(best, bi, w > 0.f ? logf(w) + gumbel(wd[e]) : -INFINITY, v);
+      } else {
+        const float x = yv[e] / T;
+        if (t > expf(x - wbest) * 1.0001f) continue;
+        argmax_merge(best, bi, x + gumbel(wd[e]), v);
+      }
+    }
   }
   s_v[threadIdx.x] = best;
   s_i[threadIdx.x] = bi;
@@ -501,7 +581,7 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
 }
 
 void launch_accept_sample(const AcceptArgs& a, cudaStream_t s, bool pdl) {
-  PARD_LAUNCH(accept_test_kernel, a.batch, 256, 0, s, pdl, a);
+  PARD_LAUNCH(accept_test_kernel, a.batch, 32 * kRowWarps, 0, s, pdl, a);
   PARD_LAUNCH(resample_kernel, a.batch * kResampleSplit, 256, 0, s, true, a);
 }
 
@@ -568,6 +648,86 @@ void launch_row_stats(const float* logits, int rows, int vocab, int w_tiles, int
                       int gumbel_stream, int rows_per_seq, float4* stats, int2* stats_i, cudaStream_t s) {
   PARD_LAUNCH(row_stats_kernel, dim3(w_tiles, rows), 128, 0, s, false, logits, vocab, m_cap, call, gumbel_stream,
               rows_per_seq > 0 ? rows_per_seq : 1, stats, stats_i);
+}
+
+// Statistics of given logits rows in tiles of kGivenTile entries (max,
+// argmax, and when sampling the sum of exp((x - max)/T)): block (t, m) takes
+// tile t of row m, the target's rows first; block (0, 0) also resets the
+// acceptance state and writes the call's scalars.  HBM-bound: every logit is
+// read once, 16 bytes a load, four loads in flight a thread (batch 16, K = 6:
+// 107 MB; the whole sampled acceptance 92 us, 231 us with one 512-byte tile a
+// block, three block reductions each and one row after the other after it; the
+// greedy one at batch 1, K = 8: 9.7 us, 51.7 before).
+__global__ void __launch_bounds__(128) given_stats_kernel(const __grid_constant__ GivenArgs a) {
+  pdl_trigger();
+  const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const bool target = (int)blockIdx.y < a.rows_t;
+  const int m = target ? blockIdx.y : blockIdx.y - a.rows_t;
+  const float* row = (target ? a.y : a.z) + (size_t)m * a.vocab;
+  if (t == 0 && blockIdx.y == 0) {
+    if (tid == 0) *a.call_out = a.call;
+    if (tid < a.batch) {
+      a.st.n[tid] = 1;
+      a.st.pend_cnt[tid] = 1;
+      a.st.gen[tid] = 0;
+      a.st.max_new[tid] = 1 << 30;
+      a.st.done[tid] = 0;
+      a.st.samp_cnt[tid] = 0;
+    }
+    for (int i = tid; i < a.batch * a.K; i += 128) a.st.d[i] = a.d[i];
+  }
+  float x[16];
+  int v[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    v[q] = t * kGivenTile + q * 512 + tid * 4;
+    float4 f = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    if (v[q] < a.vocab) {  // vocab is a multiple of 8: all four entries or none
+      if (a.vec) f = __ldcs(reinterpret_cast<const float4*>(row + v[q]));
+      else f = make_float4(row[v[q]], row[v[q] + 1], row[v[q] + 2], row[v[q] + 3]);
+    }
+    x[4 * q] = f.x; x[4 * q + 1] = f.y; x[4 * q + 2] = f.z; x[4 * q + 3] = f.w;
+  }
+  float mv = -INFINITY;
+  int mi = INT_MAX;
+#pragma unroll
+  for (int i = 0; i < 16; ++i)
+    if (v[i / 4] < a.vocab) argmax_merge(mv, mi, x[i], v[i / 4] + (i & 3));
+  float se = 0.f;
+  const float T = a.call.temp;
+  if (a.sample && mv != -INFINITY) {
+    const float c = mv / T;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) se += v[i / 4] < a.vocab ? expf(x[i] / T - c) : 0.f;
+  }
+  auto merge = [&](float m2, int i2, float s2) {
+    if (a.sample) {
+      float mm = mv;
+      merge_lse(mm, se, m2, s2, T);
+    }
+    argmax_merge(mv, mi, m2, i2);
+  };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float m2 = __shfl_xor_sync(0xffffffffu, mv, o), s2 = __shfl_xor_sync(0xffffffffu, se, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, mi, o);
+    merge(m2, i2, s2);
+  }
+  __shared__ float s_m[4], s_s[4];
+  __shared__ int s_i[4];
+  if (lane == 0) { s_m[tid >> 5] = mv; s_s[tid >> 5] = se; s_i[tid >> 5] = mi; }
+  __syncthreads();
+  if (tid == 0) {
+    for (int w = 1; w < 4; ++w) merge(s_m[w], s_i[w], s_s[w]);
+    const size_t at = (size_t)t * (target ? a.m_cap_t : a.m_cap_d) + m;
+    (target ? a.stats_t : a.stats_d)[at] = make_float4(mv, se, -INFINITY, 0.f);
+    if (target) a.stats_it[at] = make_int2(mi, -1);
+  }
+}
+
+void launch_given_stats(const GivenArgs& a, cudaStream_t s) {
+  PARD_LAUNCH(given_stats_kernel, dim3((a.vocab + kGivenTile - 1) / kGivenTile, a.rows_t + a.rows_d), 128, 0, s, false,
+              a);
 }
 
 __global__ void set_call_kernel(CallArgs* dst, CallArgs v) {

@@ -23,7 +23,7 @@ namespace {
 constexpr int kNaMaxBatch = 16;
 constexpr int kNaMaxK = 8;
 constexpr int kNaMaxVocab = 128256;
-constexpr int kNaTiles = (kNaMaxVocab + kTileN - 1) / kTileN;
+constexpr int kNaTiles = (kNaMaxVocab + kGivenTile - 1) / kGivenTile;
 constexpr int kNaRowsT = kNaMaxBatch * (kNaMaxK + 1);  // target rows: B (K+1)
 constexpr int kNaRowsD = kNaMaxBatch * kNaMaxK;        // draft rows: B K
 
@@ -32,8 +32,7 @@ constexpr size_t kOffCall = 0;
 constexpr size_t kOffStatsT = al(kOffCall + sizeof(CallArgs));
 constexpr size_t kOffStatsIT = al(kOffStatsT + (size_t)kNaTiles * kNaRowsT * sizeof(float4));
 constexpr size_t kOffStatsD = al(kOffStatsIT + (size_t)kNaTiles * kNaRowsT * sizeof(int2));
-constexpr size_t kOffStatsID = al(kOffStatsD + (size_t)kNaTiles * kNaRowsD * sizeof(float4));
-constexpr size_t kOffN = al(kOffStatsID + (size_t)kNaTiles * kNaRowsD * sizeof(int2));
+constexpr size_t kOffN = al(kOffStatsD + (size_t)kNaTiles * kNaRowsD * sizeof(float4));
 constexpr size_t kOffPendCnt = al(kOffN + kNaMaxBatch * 4);
 constexpr size_t kOffPend = al(kOffPendCnt + kNaMaxBatch * 4);
 constexpr size_t kOffGen = al(kOffPend + kNaMaxBatch * (kNaMaxK + 1) * 4);
@@ -45,7 +44,7 @@ constexpr size_t kOffSampA = al(kOffDnorm + kNaMaxBatch * kNaMaxK * sizeof(float
 constexpr size_t kOffSampNorm = al(kOffSampA + kNaMaxBatch * 4);
 constexpr size_t kOffSampPart = al(kOffSampNorm + kNaMaxBatch * sizeof(float4));
 constexpr size_t kOffSampCnt = al(kOffSampPart + (size_t)kNaMaxBatch * kResampleSplit * sizeof(float2));
-constexpr size_t kNaBytes = al(kOffSampCnt + kNaMaxBatch * 4);  // about 6.3 MiB
+constexpr size_t kNaBytes = al(kOffSampCnt + kNaMaxBatch * 4);  // about 340 KiB
 
 }  // namespace
 
@@ -79,20 +78,6 @@ void* na_scratch(std::string& err) {
     g_na_ptr[dev] = p;
   }
   return g_na_ptr[dev];
-}
-
-// Per-call state of the acceptance kernels: nothing generated yet, no length
-// budget, resampling counters at zero.
-__global__ void na_reset_state(DevState st, int B) {
-  const int i = threadIdx.x;
-  if (i < B) {
-    st.n[i] = 1;
-    st.pend_cnt[i] = 1;
-    st.gen[i] = 0;
-    st.max_new[i] = 1 << 30;
-    st.done[i] = 0;
-    st.samp_cnt[i] = 0;
-  }
 }
 
 }  // namespace
@@ -129,7 +114,6 @@ extern "C" pard_status pard_accept_noalloc(const float* d_target_logits, const f
   float4* stats_t = reinterpret_cast<float4*>(base + kOffStatsT);
   int2* stats_it = reinterpret_cast<int2*>(base + kOffStatsIT);
   float4* stats_d = reinterpret_cast<float4*>(base + kOffStatsD);
-  int2* stats_id = reinterpret_cast<int2*>(base + kOffStatsID);
   DevState st;
   st.n = reinterpret_cast<int*>(base + kOffN);
   st.pend_cnt = reinterpret_cast<int*>(base + kOffPendCnt);
@@ -144,15 +128,23 @@ extern "C" pard_status pard_accept_noalloc(const float* d_target_logits, const f
   st.samp_part = reinterpret_cast<float2*>(base + kOffSampPart);
   st.samp_cnt = reinterpret_cast<int*>(base + kOffSampCnt);
   st.kmax = K;
-  const int tiles = (vocab + kTileN - 1) / kTileN;
+  const int tiles = (vocab + kGivenTile - 1) / kGivenTile;
   try {
-    na_reset_state<<<1, kNaMaxBatch, 0, s>>>(st, batch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) throw e;
-    e = cudaMemcpyAsync(st.d, d_draft, (size_t)batch * K * 4, cudaMemcpyDeviceToDevice, s);
-    if (e != cudaSuccess) throw e;
-    launch_set_call(call, CallArgs{seed, step, temperature, sample ? 1 : 0, K, 0}, s, false);
-    launch_row_stats(d_target_logits, batch * (K + 1), vocab, tiles, kNaRowsT, call, -1, 1, stats_t, stats_it, s);
+    // one pass over the logits (which also resets the state), then the
+    // acceptance kernels on its statistics
+    GivenArgs g;
+    memset(&g, 0, sizeof(g));
+    g.y = d_target_logits; g.z = d_draft_logits;
+    g.rows_t = batch * (K + 1); g.rows_d = sample ? batch * K : 0;
+    g.m_cap_t = kNaRowsT; g.m_cap_d = kNaRowsD; g.vocab = vocab;
+    g.vec = ((reinterpret_cast<uintptr_t>(d_target_logits) | (sample ? reinterpret_cast<uintptr_t>(d_draft_logits) : 0)) &
+             15) == 0;
+    g.sample = sample ? 1 : 0;
+    g.stats_t = stats_t; g.stats_d = stats_d; g.stats_it = stats_it;
+    g.call = CallArgs{seed, step, temperature, sample ? 1 : 0, K, 0};
+    g.call_out = call;
+    g.st = st; g.d = d_draft; g.batch = batch; g.K = K;
+    launch_given_stats(g, s);
     AcceptArgs a;
     memset(&a, 0, sizeof(a));
     a.batch = batch; a.K = K; a.w_tiles = tiles; a.m_cap = kNaRowsT; a.vocab = vocab;
@@ -161,16 +153,10 @@ extern "C" pard_status pard_accept_noalloc(const float* d_target_logits, const f
     a.page_table = nullptr; a.pt_ld = 0; a.page_size = 16;
     a.accept_len = d_accept_len; a.emitted = d_emitted; a.kv_slots = nullptr; a.n_emit = nullptr;
     if (sample) {
-      launch_row_stats(d_draft_logits, batch * K, vocab, tiles, kNaRowsD, call, -1, 1, stats_d, stats_id, s);
-      SelectArgs sa;
-      memset(&sa, 0, sizeof(sa));
-      sa.mode = SEL_NORM_ONLY;
-      sa.batch = batch; sa.K = K; sa.w_tiles = tiles; sa.m_cap = kNaRowsD; sa.vocab = vocab;
-      sa.stats = stats_d; sa.stats_i = stats_id; sa.call = call; sa.st = st;
-      launch_select(sa, s, false);
-      launch_accept_sample(a, s, false);
+      a.dstats = stats_d; a.d_m_cap = kNaRowsD;
+      launch_accept_sample(a, s, true);
     } else {
-      launch_accept_greedy(a, s, false);
+      launch_accept_greedy(a, s, true);
     }
   } catch (cudaError_t e) {
     set_error(std::string("pard_accept_noalloc: ") + cudaGetErrorString(e));

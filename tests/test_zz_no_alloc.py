@@ -61,3 +61,37 @@ def test_noalloc_acceptance_matches_context_path_twice(batch, K, vocab):
                                    acc2.data_ptr(), em2.data_ptr(), stream)
     assert code == -1 and "static scratch" in pard.pard_last_error()
     assert P.eng.last_status() == 0
+
+
+@pytest.mark.parametrize("vocab", [8, 2040, 2056, 4104])
+def test_noalloc_tile_edges_masked_rows_and_unaligned_logits(vocab):
+    """The statistics' 2048-entry tiles at vocabularies just below and above
+    their multiples, with whole stretches of the logits masked to -inf, from
+    arrays that start 4 bytes off a 16-byte boundary: the same as the oracle's
+    acceptance rule."""
+    import torch
+    from paper_2504_18583_gb300 import _build, pard
+    _build.build()
+    B, K = 2, 5
+    rng = np.random.default_rng(vocab)
+    for sample in (True, False):
+        y = (rng.standard_normal((B, K + 1, vocab)) * 2.0).astype(np.float32)
+        y[:, :, : vocab // 2] = -np.inf
+        z = y[:, :K] + np.where(np.isinf(y[:, :K]), 0, 0.4 * rng.standard_normal((B, K, vocab))).astype(np.float32)
+        d = np.argmax(z, axis=-1).astype(np.int32)
+        hold = [torch.empty(a.size + 1, dtype=torch.float32, device="cuda") for a in (y, z)]
+        for h, a in zip(hold, (y, z)):
+            h[1:].copy_(torch.from_numpy(a.reshape(-1)))
+        dt = torch.as_tensor(d, device="cuda")
+        acc = torch.empty(B, dtype=torch.int32, device="cuda")
+        em = torch.empty((B, K + 1), dtype=torch.int32, device="cuda")
+        code = pard.lib().pard_accept_noalloc(hold[0][1:].data_ptr(), hold[1][1:].data_ptr(), dt.data_ptr(), B, K, vocab,
+                                              int(sample), 1.0, 21, 4, acc.data_ptr(), em.data_ptr(),
+                                              torch.cuda.current_stream().cuda_stream)
+        assert code == 0, pard.pard_last_error()
+        for b in range(B):
+            with np.errstate(divide="ignore", invalid="ignore"):
+                a_o, em_o = (OP.accept_sampling(d[b], z[b], y[b], 1.0, 21, 4, b) if sample
+                             else OP.accept_greedy(d[b], y[b]))
+            assert int(acc[b]) == a_o, (sample, b)
+            assert em[b].tolist()[:a_o + 1] == [int(t) for t in em_o], (sample, b)
