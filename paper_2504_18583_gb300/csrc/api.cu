@@ -102,9 +102,9 @@ int round_up(int x, int m) { return (x + m - 1) / m * m; }
 Dims make_dims(const pard_model_cfg& t, const pard_model_cfg& d, const pard_limits& lim, int sm) {
   Dims D;
   D.m_dec = lim.max_batch * 2 * lim.max_k;
-  // whole token tiles of the widest pass (tiles of 128 rows above 64)
+  // whole token tiles of the widest pass (tiles of up to kWideTok rows above 64)
   const int mrows = std::max(D.m_dec, lim.prefill_chunk);
-  D.MC = round_up(mrows, mrows > 64 ? 128 : 64);
+  D.MC = mrows <= 64 ? 64 : (mrows <= 128 ? 128 : round_up(mrows, kWideTok));
   // whole token tiles of the LM-head input
   D.gcap = lim.max_batch <= 16 ? 16 : (lim.max_batch <= 64 ? 64 : round_up(lim.max_batch, 128));
   D.dmax = std::max(t.d_model, d.d_model);
@@ -180,7 +180,7 @@ WsOffsets layout_ws(const Dims& D, const pard_limits& lim) {
   for (int mi = 0; mi < 2; ++mi) o.rope[mi] = L.take((size_t)D.pt_ld * lim.page_size * (D.hdmax / 2) * 8);
   o.g_plen = L.take((size_t)B * 4);
   o.mask_ids = L.take((size_t)std::max(K, 1) * 4);
-  o.gpart = L.take((size_t)D.sm * 2 * kTileN * (D.MC > 64 ? 128 : 64) * 4);  // two partial tiles per CTA
+  o.gpart = L.take((size_t)D.sm * 2 * kTileN * (D.MC > 64 ? kWideTok : 64) * 4);  // two partial tiles per CTA
   o.pack_tmp = L.take(kPackTmpBytes);
   o.total = L.total + 256;
   return o;
@@ -235,8 +235,10 @@ PFN_cuTensorMapEncodeTiled_v12000 get_encode() {
   return fn;
 }
 
-// 2-D bf16 row-major [rows][cols] tensor map, box {64 cols, box_rows}, 128B swizzle.
-CUtensorMap make_map(const void* base, int rows, int cols, int box_rows) {
+// 2-D bf16 row-major [rows][cols] tensor map, box {64 cols, box_rows}.
+// swizzled: 128-byte swizzle in shared memory (row-major operands); packed
+// operands are stored in that order already and are [rows][64] tensors.
+CUtensorMap make_map(const void* base, size_t rows, int cols, int box_rows, bool swizzled) {
   CUtensorMap m;
   std::memset(&m, 0, sizeof(m));
   auto enc = get_encode();
@@ -246,15 +248,15 @@ CUtensorMap make_map(const void* base, int rows, int cols, int box_rows) {
   cuuint32_t box[2] = {(cuuint32_t)kChunkK, (cuuint32_t)box_rows};
   cuuint32_t es[2] = {1, 1};
   CUresult r = enc(&m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) throw CudaFail{cudaErrorInvalidValue, "cuTensorMapEncodeTiled rejected a tensor"};
   return m;
 }
 
-// Token tile of a pass of up to `rows` rows: 16, 64, or 128 (65 and more
-// rows: one pass over the weights covers 128 of them).
-int pick_tt(int rows) { return rows <= 16 ? 16 : (rows <= 64 ? 64 : 128); }
+// Token tile of a pass of up to `rows` rows: 16, 64, or (more) the wide
+// kernel's, kWideTok.
+int pick_tt(int rows) { return rows <= 16 ? 16 : (rows <= 64 ? 64 : kWideTok); }
 
 }  // namespace
 
@@ -265,6 +267,10 @@ struct pard_ctx {
   WsOffsets o;
   uint8_t* ws = nullptr;
   int sm = 0;
+  int pairs = 0;          // CTA pairs of the wide GEMM the GPU holds at once
+  // activation buffers xd, xo, xf as tensors of 128-byte rows, in boxes of
+  // 16, 32, .. 256 rows (the wide GEMM's half tiles)
+  CUtensorMap xmap[3][kWideTok / 16];
   // device views
   float *h, *ssq, *ssqg, *q, *gpart, *logits, *dlogits;
   __nv_bfloat16 *xd, *xo, *xf, *xg;
@@ -307,8 +313,12 @@ void set_call(pard_ctx* c, uint64_t seed, uint64_t step, float temp, int sample,
 GemmArgs gemm_base(pard_ctx* c, int rows_cap, int tt) {
   GemmArgs a;
   std::memset(&a, 0, sizeof(a));
-  a.tok_tiles = (rows_cap + tt - 1) / tt;
-  a.n_tok = a.tok_tiles == 1 ? round_up(rows_cap, 8) : 0;
+  if (tt == kWideTok) {
+    wide_tiles(rows_cap, a.tok_tiles, a.n_tok);
+  } else {
+    a.tok_tiles = (rows_cap + tt - 1) / tt;
+    a.n_tok = a.tok_tiles == 1 ? round_up(rows_cap, 8) : 0;
+  }
   a.m_cap = c->D.MC;
   a.m_dev = c->rp.m_dev;
   a.partials = c->gpart;
@@ -319,6 +329,20 @@ GemmArgs gemm_base(pard_ctx* c, int rows_cap, int tt) {
 }
 
 void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
+  if (tt == kWideTok) {
+    const long w_pairs = (a.w_tiles + 1) / 2;
+    const long units = w_pairs * a.tok_tiles * a.kc;
+    if (2 * w_pairs * a.tok_tiles > kMaxGemmTiles || (units + 1) * (c->pairs + 1) > INT32_MAX) throw cudaErrorInvalidValue;
+    WideArgs w;
+    w.g = a;
+    const int buf = a.x == c->xd ? 0 : a.x == c->xo ? 1 : 2;
+    w.x[0] = c->xmap[buf][a.n_tok / 16 - 1];
+    w.x[1] = c->xmap[buf][kWideBoxL / 16 - 1];
+    w.x[2] = c->xmap[buf][kWideBoxS / 16 - 1];
+    launch_gemm_wide(w, wide_pairs((int)units, a.kc, c->pairs), s, true);
+    c->launches++;
+    return;
+  }
   const long U = (long)a.w_tiles * a.tok_tiles * a.kc;
   // at least 8 units (128 KB of weights) a CTA: with fewer, the split-K
   // finish of a tile gathers partials from too many CTAs; and at least
@@ -326,7 +350,7 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
   // finisher tracks their arrivals in one 64-bit mask)
   const long min_units = std::max<long>(8, (a.kc + 61) / 62);
   const int grid = (int)std::min<long>(c->sm, std::max<long>(1, U / min_units));
-  if ((long)a.w_tiles * a.tok_tiles > kMaxGemmTiles) throw cudaErrorInvalidValue;
+  if ((long)a.w_tiles * a.tok_tiles > kMaxGemmTiles || (U + 1) * (grid + 1) > INT32_MAX) throw cudaErrorInvalidValue;
   launch_gemm(a, tt, grid, s, true);
   c->launches++;
 }
@@ -381,7 +405,7 @@ struct LayerPlan {
   GemmArgs qkv, o, gu, dn;
   AttnArgs at;
 };
-LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int tt_gu, int batch, const int* pt_attn,
+LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int batch, const int* pt_attn,
                      const AttnGeom& geo, int fixed_rows) {
   Model& M = c->m[mi];
   const pard_model_cfg& cf = M.cfg;
@@ -447,7 +471,7 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int tt_gu
   // RMSNorm -> gate/up (paired 64-row tiles) -> SiLU(gate) * up
   {
     GemmArgs& a = P.gu;
-    a = gemm_base(c, rows_cap, tt_gu);
+    a = gemm_base(c, rows_cap, tt);
     a.wmap[0] = Mp.g; a.wmap[1] = Mp.u;
     a.wpk[0] = M.P[l].t[W_G]; a.wpk[1] = M.P[l].t[W_U];
     if (!a.wpk[0] || !a.wpk[1]) a.wpk[0] = a.wpk[1] = nullptr;
@@ -484,16 +508,10 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int tt_gu
 // by its sequence index.
 void run_layers(pard_ctx* c, int mi, int rows_cap, int batch, int rows_per_seq, const int* pt_attn,
                 cudaStream_t s, int fixed_rows = 0) {
-  // Above 64 rows the gate/up projection takes the 128-token tile (one pass
-  // over its weights for all rows), the QKV, O and down projections keep
-  // 64-token tiles (two passes): they have only 32-48 output tiles, so with
-  // 128-token tiles each tile's split-K finish and epilogue (8 chunks) falls
-  // on few CTAs and outlasts the bytes saved.
-  const int tt_gu = pick_tt(rows_cap);
-  const int tt = std::min(tt_gu, 64);
+  const int tt = pick_tt(rows_cap);
   const AttnGeom geo = attn_geometry(c, mi, rows_per_seq, batch);
   for (int l = 0; l < c->m[mi].cfg.n_layers; ++l) {
-    LayerPlan P = layer_plan(c, mi, l, rows_cap, tt, tt_gu, batch, pt_attn, geo, fixed_rows);
+    LayerPlan P = layer_plan(c, mi, l, rows_cap, tt, batch, pt_attn, geo, fixed_rows);
     // the pass's row count is written by the embedding kernel, which directly
     // precedes only the first QKV projection
     P.qkv.m_early = l > 0;
@@ -502,7 +520,7 @@ void run_layers(pard_ctx* c, int mi, int rows_cap, int batch, int rows_per_seq, 
     launch_attention(P.at, geo.groups * geo.n_split, s, true);
     c->launches++;
     run_gemm(c, P.o, tt, s);
-    run_gemm(c, P.gu, tt_gu, s);
+    run_gemm(c, P.gu, tt, s);
     run_gemm(c, P.dn, tt, s);
   }
 }
@@ -647,6 +665,7 @@ pard_status pard_load_weights(pard_ctx** out, const pard_model_cfg* tcfg, const 
     CK(cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev));
     if (major != 10) return fail(PARD_ERR_CUDA, "libpard is compiled for compute capability 10.x (GB300, sm_103a) only");
     c->sm = std::min(c->sm, 160);
+    c->pairs = gemm_wide_max_pairs(c->sm);
     c->lim = *lim;
     c->D = make_dims(*tcfg, *dcfg, *lim, c->sm);
     c->o = layout_ws(c->D, *lim);
@@ -671,6 +690,14 @@ pard_status pard_load_weights(pard_ctx** out, const pard_model_cfg* tcfg, const 
     c->call = c->at<CallArgs>(o.call); c->status = c->at<uint32_t>(o.status);
     c->paths = c->at<uint32_t>(o.paths);
 
+    {
+      const __nv_bfloat16* buf[3] = {c->xd, c->xo, c->xf};
+      const int cols[3] = {c->D.dmax, c->D.qdmax, c->D.ffn_pad};
+      if (c->D.MC > 64)  // the wide GEMM's passes
+        for (int i = 0; i < 3; ++i)
+          for (int k = 0; k < kWideTok / 16; ++k)
+            c->xmap[i][k] = make_map(buf[i], (size_t)(cols[i] / 64) * 2 * c->D.MC, 64, 16 * (k + 1), false);
+    }
     c->tmp_pos = c->at<int>(o.tmp_pos); c->g_plen = c->at<int>(o.g_plen);
     c->mask_ids = c->at<int>(o.mask_ids);
 
@@ -698,16 +725,7 @@ pard_status pard_load_weights(pard_ctx** out, const pard_model_cfg* tcfg, const 
       const int d = M.cfg.d_model, qd = M.qd(), kvd = M.kvd(), ffn = M.cfg.ffn;
       for (int l = 0; l < M.cfg.n_layers; ++l) {
         for (int j = 0; j < 9; ++j) M.L[l].t[j] = reinterpret_cast<const __nv_bfloat16*>(W[mi]->layers[l * 9 + j]);
-        LayerMaps& mp = M.maps[l];
-        mp.q = make_map(M.L[l].t[W_Q], qd, d, kTileN);
-        mp.k = make_map(M.L[l].t[W_K], kvd, d, kTileN);
-        mp.v = make_map(M.L[l].t[W_V], kvd, d, kTileN);
-        mp.o = make_map(M.L[l].t[W_O], d, qd, kTileN);
-        mp.g = make_map(M.L[l].t[W_G], ffn, d, 64);
-        mp.u = make_map(M.L[l].t[W_U], ffn, d, 64);
-        mp.dn = make_map(M.L[l].t[W_D], d, ffn, kTileN);
       }
-      M.lm_map = make_map(M.lm_head, M.cfg.vocab, d, kTileN);
       // pack every matrix whose shape allows it, in place (each matrix once,
       // also when the draft shares the target's tensors)
       M.P.assign(M.cfg.n_layers, LayerW{});
@@ -721,9 +739,14 @@ pard_status pard_load_weights(pard_ctx** out, const pard_model_cfg* tcfg, const 
         }
         return w;
       };
+      // the matrix's tensor map, packed or row-major, boxes of R rows
+      auto map_of = [&](const __nv_bfloat16* w, const __nv_bfloat16* pk, int N, int K, int R) {
+        return pk ? make_map(pk, (size_t)N * (K / 64), 64, R, false) : make_map(w, N, K, R, true);
+      };
       for (int l = 0; l < M.cfg.n_layers; ++l) {
         const LayerW& Wl = M.L[l];
         LayerW& Pl = M.P[l];
+        LayerMaps& mp = M.maps[l];
         for (int j = 0; j < 9; ++j) Pl.t[j] = nullptr;
         Pl.t[W_Q] = pack(Wl.t[W_Q], qd, d, kTileN);
         Pl.t[W_K] = pack(Wl.t[W_K], kvd, d, kTileN);
@@ -734,8 +757,16 @@ pard_status pard_load_weights(pard_ctx** out, const pard_model_cfg* tcfg, const 
           Pl.t[W_U] = pack(Wl.t[W_U], ffn, d, 64);
         }
         Pl.t[W_D] = pack(Wl.t[W_D], d, ffn, kTileN);
+        mp.q = map_of(Wl.t[W_Q], Pl.t[W_Q], qd, d, kTileN);
+        mp.k = map_of(Wl.t[W_K], Pl.t[W_K], kvd, d, kTileN);
+        mp.v = map_of(Wl.t[W_V], Pl.t[W_V], kvd, d, kTileN);
+        mp.o = map_of(Wl.t[W_O], Pl.t[W_O], d, qd, kTileN);
+        mp.g = map_of(Wl.t[W_G], Pl.t[W_G], ffn, d, 64);
+        mp.u = map_of(Wl.t[W_U], Pl.t[W_U], ffn, d, 64);
+        mp.dn = map_of(Wl.t[W_D], Pl.t[W_D], d, ffn, kTileN);
       }
       M.lm_pk = pack(M.lm_head, M.cfg.vocab, d, kTileN);
+      M.lm_map = map_of(M.lm_head, M.lm_pk, M.cfg.vocab, d, kTileN);
       CK(cudaStreamSynchronize(s));
       M.kv = reinterpret_cast<__nv_bfloat16*>(kvp);
       M.n_pages_ = lim->n_pages;

@@ -176,9 +176,9 @@ __global__ void __launch_bounds__(kAttnThreads) attn_kernel(const __grid_constan
     __nv_bfloat16 h0, l0, h1, l1;
     split_bf16(acc.x / L, h0, l0);
     split_bf16(acc.y / L, h1, l1);
-    *reinterpret_cast<uint32_t*>(a.x_out + xpk(2 * m, col, a.x_rows)) =
+    *reinterpret_cast<uint32_t*>(a.x_out + xpk(m, 0, col, a.x_rows)) =
         (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    *reinterpret_cast<uint32_t*>(a.x_out + xpk(2 * m + 1, col, a.x_rows)) =
+    *reinterpret_cast<uint32_t*>(a.x_out + xpk(m, 1, col, a.x_rows)) =
         (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
   }
   cluster_sync();  // peers may still be reading this CTA's partial

@@ -6,8 +6,8 @@
 //  * operand swap: the weight tile is the UMMA A operand (M = 128 weight
 //    rows), the activations the B operand (N = 2 x token tile), so a skinny
 //    M=9 product still issues full 128-row tensor-core tiles;
-//  * activations are carried as bf16 hi/lo pairs (x = hi + lo, rows 2m and
-//    2m+1 of the B operand), which keeps fp32-level accuracy of the products
+//  * activations are carried as bf16 hi/lo pairs (x = hi + lo, each a row of
+//    the B operand), which keeps fp32-level accuracy of the products
 //    with bf16 tensor-core inputs; hi and lo columns are summed in the
 //    epilogue;
 //  * warp 0 streams 128x64 weight tiles and the matching activation tile
@@ -30,7 +30,7 @@
 
 namespace pard {
 
-template <int TT>
+template <int TT, int MODE>
 // two CTAs per SM at the 16-token tile: this launch's and the next one's
 __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __grid_constant__ GemmArgs a) {
   using C = GemmCfg<TT>;
@@ -61,10 +61,10 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   int* live = reinterpret_cast<int*>(misc + 4);  // [0] token tiles processed, [1] token rows of one tile's MMA
   // this CTA's units (recomputed below in the rare launch that drops token tiles)
   const bool early = a.m_early && a.tok_tiles > 1;
-  const long G = gridDim.x;
-  const long c = blockIdx.x;
-  long U = (long)a.w_tiles * a.tok_tiles * a.kc;
-  long u0 = range_start(c, U, G), u1 = range_start(c + 1, U, G);
+  const int G = gridDim.x;
+  const int c = blockIdx.x;
+  int U = a.w_tiles * a.tok_tiles * a.kc;
+  int u0 = range_start(c, U, G), u1 = range_start(c + 1, U, G);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   const uint32_t tmem = *tmem_slot;
   const int tok_tiles = early ? live[0] : a.tok_tiles;
   if (tok_tiles != a.tok_tiles) {
-    U = (long)a.w_tiles * tok_tiles * a.kc;
+    U = a.w_tiles * tok_tiles * a.kc;
     u0 = range_start(c, U, G);
     u1 = range_start(c + 1, U, G);
   }
@@ -116,13 +116,13 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
       const uint64_t pol = policy_evict_first();
       for (int i = 0; i < kMaxSeg; ++i)
         if ((i < a.nseg || (a.pair && i < 2)) && !a.wpk[i]) tma_prefetch_desc(&a.wmap[i]);
-      const int n = (int)(u1 - u0);
+      const int n = u1 - u0;
       const int npre = n < P ? n : P;
       // Unit cursor advanced incrementally: the producer issues one stage per
       // wake-up with no divisions on the path between the 'empty' signal and
       // the copies.
-      int kk = (int)(u0 % a.kc);
-      int w_tile = (int)((u0 / a.kc) / tok_tiles), tok_tile = (int)((u0 / a.kc) % tok_tiles);
+      int kk = u0 % a.kc;
+      int w_tile = u0 / a.kc / tok_tiles, tok_tile = u0 / a.kc % tok_tiles;
       const __nv_bfloat16* wsrc0 = nullptr;  // packed block base of the current weight tile (A)
       const __nv_bfloat16* wsrc1 = nullptr;  // second half (gate/up pairs)
       const CUtensorMap* wmap0 = nullptr;
@@ -210,9 +210,9 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
       uint32_t fph = 0;   // its 'full' phase parity
       int seg_i = 0;
       bool ok = true;
-      for (long u = u0; u < u1 && ok;) {
-        const long t = u / a.kc;
-        const long ub = u, ue = (t + 1) * a.kc < u1 ? (t + 1) * a.kc : u1;
+      for (int u = u0; u < u1 && ok;) {
+        const int t = u / a.kc;
+        const int ub = u, ue = (t + 1) * a.kc < u1 ? (t + 1) * a.kc : u1;
         const int ab = seg_i % C::kNumAcc;
         const uint32_t aph = (uint32_t)((seg_i / C::kNumAcc) & 1) ^ 1u;
         if (!mbar_wait(&acce[ab], aph, abort_flag)) { ok = false; break; }
@@ -251,21 +251,21 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
     }
     int seg_i = 0;
     int rs_tok = -1;  // token tile whose RMS row scale S.rs holds
-    for (long u = u0; u < u1;) {
-      const long t = u / a.kc;
-      const long ub = u, ue = (t + 1) * a.kc < u1 ? (t + 1) * a.kc : u1;
+    for (int u = u0; u < u1;) {
+      const int t = u / a.kc;
+      const int ub = u, ue = (t + 1) * a.kc < u1 ? (t + 1) * a.kc : u1;
       u = ue;
       const int ab = seg_i % C::kNumAcc;
-      const int w_tile = (int)(t / tok_tiles), tok_tile = (int)(t % tok_tiles);
+      const int w_tile = t / tok_tiles, tok_tile = t % tok_tiles;
       const int tok_base = tok_tile * TT;
-      if (a.ssq_in && tok_base != rs_tok) {
+      if (MODE != MODE_RESID && tok_base != rs_tok) {
         epi_row_scale<TT>(a, tok_base, et, M, S);
         rs_tok = tok_base;
       }
       // result-independent loads of a segment this CTA finishes (it starts
       // the tile), issued while the MMAs run
       EpiPre pre0 = {};
-      if (ub == t * a.kc) pre0 = epi_pre(a, w_tile, tok_base, et, M);
+      if (ub == t * a.kc) pre0 = epi_pre<MODE>(a, w_tile, tok_base, et, M);
       if (!mbar_wait(&accf[ab], (uint32_t)((seg_i / C::kNumAcc) & 1), abort_flag)) {
         if (et == 0) set_status(a.status, ST_TIMEOUT_EPI);
         *abort_flag = 1;
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
       tc_fence_after();
       epi_bar();
       const uint32_t tbase = tmem + ab * C::kAccCols + ((uint32_t)(q * 32) << 16);
-      if (!epi_segment_owned<TT>(a, t, ub, ue, u0, U, G, c, tbase, w_tile, tok_base, fr, et, M, S, pre0,
+      if (!epi_segment_owned<TT, MODE>(a, t, ub, ue, u0, U, G, c, tbase, w_tile, tok_base, fr, et, M, S, pre0,
                                  reinterpret_cast<float*>(sA), (uint32_t)(C::kStages * C::kStageBytes), fx,
                                  fx_armed, abort_flag, bcast))
         break;
@@ -307,21 +307,12 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   }
 }
 
-int gemm_smem_bytes(int tt) {
-  switch (tt) {
-    case 16: return GemmCfg<16>::kSmem;
-    case 64: return GemmCfg<64>::kSmem;
-    case 128: return GemmCfg<128>::kSmem;
-    default: return -1;
-  }
-}
-
-template <int TT>
+template <int TT, int MODE>
 static cudaError_t launch_tt(const GemmArgs& a, int grid, cudaStream_t s, bool pdl) {
   static bool configured = false;
   const int smem = GemmCfg<TT>::kSmem;
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<TT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<TT, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     configured = true;
   }
@@ -335,16 +326,21 @@ static cudaError_t launch_tt(const GemmArgs& a, int grid, cudaStream_t s, bool p
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gemm_kernel<TT>, a);
+  return cudaLaunchKernelEx(&cfg, gemm_kernel<TT, MODE>, a);
+}
+
+template <int TT>
+static cudaError_t launch_mode(const GemmArgs& a, int grid, cudaStream_t s, bool pdl) {
+  switch (a.mode) {
+    case MODE_QKV: return launch_tt<TT, MODE_QKV>(a, grid, s, pdl);
+    case MODE_RESID: return launch_tt<TT, MODE_RESID>(a, grid, s, pdl);
+    case MODE_SWIGLU: return launch_tt<TT, MODE_SWIGLU>(a, grid, s, pdl);
+    default: return launch_tt<TT, MODE_LOGITS>(a, grid, s, pdl);
+  }
 }
 
 void launch_gemm(const GemmArgs& a, int tt, int grid, cudaStream_t s, bool pdl) {
-  cudaError_t e;
-  switch (tt) {
-    case 16: e = launch_tt<16>(a, grid, s, pdl); break;
-    case 64: e = launch_tt<64>(a, grid, s, pdl); break;
-    default: e = launch_tt<128>(a, grid, s, pdl); break;
-  }
+  const cudaError_t e = tt == 16 ? launch_mode<16>(a, grid, s, pdl) : launch_mode<64>(a, grid, s, pdl);
   if (e != cudaSuccess) throw e;
 }
 

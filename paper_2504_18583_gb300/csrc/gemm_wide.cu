@@ -1,0 +1,598 @@
+// GEMM of passes with more than 64 rows: batched decoding (112 verify rows at
+// batch 16) and prompt passes (up to a whole prefill chunk).
+//
+// At these sizes a weight tile meets so many tokens that the traffic into the
+// SMs bounds a kernel, not HBM: a CTA that multiplies 128 weight rows with 128
+// tokens (hi and lo parts: 32 KB a 64-column step) takes 48 KB from L2 per
+// 16 KB of weights.  Here a pair of CTAs (cta_group::2) shares a tile of 256
+// weight rows and up to 256 tokens: each CTA loads its own 128 weight rows
+// and half of the tokens, the tensor cores read the other half from the peer.
+// The hi and lo parts of a token go to the same accumulator column (two MMAs
+// per 16 columns of K, selected by the descriptors' atom stride), which
+// halves the accumulator: two 256-column buffers, so one tile's epilogue runs
+// under the next tile's MMAs.
+//
+// The (tile, K-step) space is split evenly over the pairs.  A tile split
+// between several pairs is finished by all of them: each stores its partial,
+// then finishes its own share of the tile's 16-token chunks, summing the
+// partials in pair order (deterministic).  (One finisher per tile gathers all
+// partials of up to 128 KB each on one SM, which took longer than the
+// multiplication.)  A pair waits for the others only after its last unit is
+// multiplied and stored, so no wait closes a circle.
+//
+// Roles per CTA: warp 0 streams, counting both CTAs' bytes on rank 0's
+// barriers (TMA tensor copies can do that; the packed operands are tensors of
+// 128-byte rows to them), warp 1 of rank 0 issues the MMAs, warps 2-5 and 6-9
+// are two epilogue groups that take alternate chunks.
+#include "gemm_core.cuh"
+
+namespace pard {
+
+namespace {
+
+constexpr int kWideRing = 192 * 1024;  // stage ring; the stages' number follows from their size
+constexpr int kWideMaxStages = 8;
+constexpr int kWideThreads = 320;
+constexpr int kWideBarBytes = (8 * (2 * kWideMaxStages + 6) + 15) / 16 * 16;
+constexpr int kWideMiscBytes = 64;
+constexpr int kWideGroupFloats = kEpiTok * kTileN + 3 * kEpiTok;  // exchange and row facts of one epilogue group
+constexpr int kWideSmem =
+    1024 + kWideRing + kWideBarBytes + kWideMiscBytes + 4 * (kWideMaxRows + 2 * kWideGroupFloats);
+static_assert(kWideSmem <= 227 * 1024, "shared memory of one CTA");
+static_assert(kWideGroupFloats % 4 == 0 && kWideMaxRows % 4 == 0 && kWideBarBytes % 16 == 0, "16-byte exchange reads");
+
+__device__ __forceinline__ void all_epi_bar() { asm volatile("bar.sync 3, 256;" ::: "memory"); }
+
+// all_epi_bar that also returns whether any of the 256 threads passed true
+__device__ __forceinline__ bool all_epi_any(bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.or.pred q, 3, 256, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"((uint32_t)v)
+      : "memory");
+  return r != 0;
+}
+
+// Epilogue values of one 16-token chunk straight from the accumulator
+__device__ __forceinline__ void load_acc(uint32_t taddr, float (&v)[kEpiTok]) {
+  uint32_t r[16];
+  tmem_ld16(taddr, r);
+#pragma unroll
+  for (int j = 0; j < kEpiTok; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+}  // namespace
+
+template <int MODE>
+__global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid_constant__ WideArgs w) {
+  const GemmArgs& a = w.g;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + kWideRing);  // rank 0: both CTAs' stage has landed
+  uint64_t* empty = full + kWideMaxStages;
+  uint64_t* accf = empty + kWideMaxStages;
+  uint64_t* acce = accf + 2;                 // rank 0: both CTAs' epilogue groups are done with the buffer
+  uint64_t* drain = acce + 2;
+  uint64_t* fx = drain + 1;                  // split tiles: partials copied into the idle ring
+  uint32_t* misc = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(full) + kWideBarBytes);
+  uint32_t* tmem_slot = misc;
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 1);
+  int* bcast = reinterpret_cast<int*>(misc + 2);
+  volatile int* fx_armed = reinterpret_cast<volatile int*>(misc + 3);  // rounds of copies issued
+  int* live = reinterpret_cast<int*>(misc + 4);  // [0] token tiles, [1] tokens a tile
+  float* rs = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(misc) + kWideMiscBytes);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const int c = blockIdx.x >> 1;  // this pair
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kWideMaxStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) { mbar_init(&accf[b], 1); mbar_init(&acce[b], 4); }
+    mbar_init(drain, 1);
+    mbar_init(fx, 1);
+    *fx_armed = 0;
+    *abort_flag = 0;
+    // A row count written two or more launches back is read now, and the
+    // tiles past it are neither loaded nor multiplied.
+    int tiles = a.tok_tiles, n_tok = a.n_tok;
+    if (a.m_early) wide_tiles(min(max(__ldcg(a.m_dev), 1), a.m_cap), tiles, n_tok);
+    live[0] = tiles;
+    live[1] = n_tok;
+    fence_barrier_init();
+  }
+  __syncthreads();
+  if (warp == 1) tmem_alloc2(tmem_slot, 512);
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // the peer's barriers are initialised before anything arrives on them
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const int tok_tiles = live[0], n_tok = live[1];
+  const int kc = a.kc;
+  // unit indices: 32 bits (the host checks that U times the pairs fits; 64-bit
+  // divisions made up half of a short launch's tail)
+  const int U = (a.w_tiles + 1) / 2 * tok_tiles * kc;
+  const int G = wide_pairs(U, kc, (int)(gridDim.x >> 1));  // pairs with work
+  auto start_of = [&](int cc) { return cc * U / G; };
+  auto owner = [&](int u) { return ((u + 1) * G + U - 1) / U - 1; };
+  const int u0 = c < G ? start_of(c) : 0, u1 = c < G ? start_of(c + 1) : 0;
+  const uint32_t b_bytes = (uint32_t)n_tok * 128;  // half of the tile's tokens, hi and lo rows
+  const uint32_t stage_bytes = (uint32_t)kTileN * 128 + b_bytes;
+  const int R = min(kWideMaxStages, kWideRing / (int)stage_bytes);
+  uint32_t armed = 0, armed_odd = 0;  // producer: slots armed at least once, and those armed an odd number of times
+
+  if (warp == 0) {
+    // ---------------- producer: this CTA's weight rows and half of the tokens ----------------
+    // The whole warp runs the loop and one elected thread issues: in a loop
+    // inside "if (lane == 0)" each copy took about 150 clocks to issue.
+    if (u1 > u0) {
+      // the weights are read again for every further token tile
+      const uint64_t pol = tok_tiles == 1 ? policy_evict_first() : policy_evict_normal();
+      if (elect_one()) {
+        for (int i = 0; i < (a.pair ? 2 : a.nseg); ++i) tma_prefetch_desc(&a.wmap[i]);
+        for (int i = 0; i < 3; ++i) tma_prefetch_desc(&w.x[i]);
+      }
+      const int n = u1 - u0;
+      const int npre = min(n, R);
+      int kk = u0 % kc;
+      int wp = u0 / kc / tok_tiles, tok_tile = u0 / kc % tok_tiles;
+      // coordinates of the current weight tile's step kk: (col0 + kk colstep, row0 + kk rowstep)
+      const CUtensorMap *wmap0 = nullptr, *wmap1 = nullptr;
+      int row0 = 0, rowstep = 0, colstep = 0;
+      auto set_tile = [&]() {
+        // an odd last tile is loaded by both CTAs and finished by rank 0 alone
+        const int w_tile = min(2 * wp + (int)rank, a.w_tiles - 1);
+        const int seg = a.pair ? 0 : seg_of(a, w_tile);
+        const int blk = a.pair ? w_tile : w_tile - a.seg_tile0[seg];
+        const int rows = a.pair ? 64 : kTileN;
+        wmap0 = &a.wmap[seg];
+        wmap1 = &a.wmap[1];
+        const bool packed = a.wpk[seg] != nullptr;  // blocks of [rows][64] in steps of K
+        row0 = packed ? blk * kc * rows : blk * rows;
+        rowstep = packed ? rows : 0;
+        colstep = packed ? 0 : kChunkK;
+      };
+      set_tile();
+      const uint64_t polx = policy_evict_normal();
+      const uint32_t full0 = mapa_shared(full, 0);  // rank 0's barriers
+      auto issue_a = [&](int s) {
+        uint8_t* dst = ring + (uint32_t)s * stage_bytes;
+        const uint32_t bar = full0 + 8 * s;
+        tma2_load_2d_hint(dst, wmap0, bar, kk * colstep, row0 + kk * rowstep, pol);
+        if (a.pair) tma2_load_2d_hint(dst + kTileN * 64, wmap1, bar, kk * colstep, row0 + kk * rowstep, pol);
+      };
+      // this rank's half of a token tile: n_tok rows of 128 bytes
+      auto issue_b = [&](int s, int kk_, int tok_) {
+        uint8_t* dst = ring + (uint32_t)s * stage_bytes + kTileN * 128;
+        const uint32_t bar = full0 + 8 * s;
+        const int row = kk_ * a.x_rows + (2 * tok_ + (int)rank) * n_tok;
+        if (n_tok == a.n_tok) {
+          tma2_load_2d_hint(dst, &w.x[0], bar, 0, row, polx);
+        } else {  // fewer rows than the launch was sized for
+          int r = 0;
+          for (; r + kWideBoxL <= n_tok; r += kWideBoxL) tma2_load_2d_hint(dst + r * 128, &w.x[1], bar, 0, row + r, polx);
+          for (; r < n_tok; r += kWideBoxS) tma2_load_2d_hint(dst + r * 128, &w.x[2], bar, 0, row + r, polx);
+        }
+      };
+      auto arm = [&](int s) {  // armed, armed_odd: by every thread of the warp
+        armed |= rank == 0 ? 1u << s : 0u;
+        armed_odd ^= rank == 0 ? 1u << s : 0u;
+      };
+      auto expect = [&](int s) {
+        if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * stage_bytes);
+      };
+      auto advance = [&]() {
+        if (++kk == kc) {
+          kk = 0;
+          if (++tok_tile == tok_tiles) { tok_tile = 0; ++wp; }
+          set_tile();
+        }
+      };
+      // weights first: they do not depend on the previous kernel
+      const int kk0 = kk, tok0 = tok_tile;
+      for (int i = 0; i < npre; ++i) {
+        arm(i);
+        if (elect_one()) {
+          expect(i);
+          issue_a(i);
+        }
+        __syncwarp();
+        advance();
+      }
+      pdl_wait();
+      for (int i = 0, k2 = kk0, t2 = tok0; i < npre; ++i) {
+        if (elect_one()) issue_b(i, k2, t2);
+        __syncwarp();
+        if (++k2 == kc) { k2 = 0; if (++t2 == tok_tiles) t2 = 0; }
+      }
+      int s = npre % R;
+      uint32_t ph = (uint32_t)((npre / R) & 1) ^ 1u;
+      for (int i = npre; i < n; ++i) {
+        if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort_flag))) {
+          if (lane == 0) set_status(a.status, ST_TIMEOUT_TMA);
+          *abort_flag = 1;
+          break;
+        }
+        arm(s);
+        if (elect_one()) {
+          expect(s);
+          issue_a(s);
+          issue_b(s, kk, tok_tile);
+        }
+        __syncwarp();
+        advance();
+        if (++s == R) { s = 0; ph ^= 1u; }
+      }
+    }
+    if (lane == 0) pdl_trigger();
+  } else if (warp == 1) {
+    if (rank == 0) {
+      // ---------------- MMA issuer of the pair: the whole warp runs the loop, one thread issues ----------------
+      // (a loop inside "if (lane == 0)" took about 100 clocks an MMA to issue)
+      const uint32_t idesc = idesc_bf16(2 * kTileN, n_tok);
+      int s = 0;
+      uint32_t fph = 0;
+      int seg_i = 0;
+      bool ok = true;
+      for (int u = u0; u < u1 && ok;) {
+        const int ub = u, ue = min((u / kc + 1) * kc, u1);
+        const int ab = seg_i & 1;
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&acce[ab], (uint32_t)((seg_i >> 1) & 1) ^ 1u, abort_flag));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d = tmem + ab * kWideTok;
+        for (; u < ue; ++u) {
+          ok = __all_sync(0xffffffffu, mbar_wait(&full[s], fph, abort_flag));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t sa = smem_u32(ring) + (uint32_t)s * stage_bytes;
+          const uint64_t ad = sw128_desc(sa);
+          const uint64_t bh = sw128_desc(sa + kTileN * 128, 2048), bl = sw128_desc(sa + kTileN * 128 + 1024, 2048);
+          if (elect_one()) {
+#pragma unroll
+            for (int k = 0; k < kChunkK / 16; ++k) {
+              umma2_bf16(d, ad + 2 * k, bh + 2 * k, idesc, (u > ub || k > 0) ? 1u : 0u);
+              umma2_bf16(d, ad + 2 * k, bl + 2 * k, idesc, 1u);
+            }
+            umma2_commit(&empty[s], 3);
+            if (u + 1 == ue) umma2_commit(&accf[ab], 3);
+          }
+          __syncwarp();
+          if (++s == R) { s = 0; fph ^= 1u; }
+        }
+        ++seg_i;
+      }
+      if (!ok && lane == 0) {
+        set_status(a.status, ST_TIMEOUT_MMA);
+        *abort_flag = 1;
+      }
+    }
+  } else {
+    // ---------------- epilogue: two groups of 128 threads ----------------
+    pdl_wait();
+    const int et256 = threadIdx.x - 64, grp = et256 >> 7, et = et256 & 127;
+    const int q = warp & 3, fr = q * 32 + lane;
+    EpiSmem S;
+    S.rs = rs;
+    S.xch = rs + kWideMaxRows + grp * kWideGroupFloats;
+    S.ri = reinterpret_cast<int*>(S.xch + kEpiTok * kTileN);
+    S.bar = 1 + grp;
+    int M = *a.m_dev;
+    if (M > a.m_cap) {
+      if (et256 == 0) set_status(a.status, ST_BAD_ROWS);
+      M = a.m_cap;
+    }
+    constexpr int kTileF = kTileN * kWideTok;  // floats of one partial tile of one CTA
+    constexpr int kChF = kTileN * kEpiTok;
+    constexpr int kRingChunks = kWideRing / (kChF * 4);  // chunks the ring holds; more contributors are read from L2
+    // RMS scales of all the pass's rows: a thread a token, its partial sums
+    // requested sixteen at a time and added in tile order
+    if constexpr (MODE != MODE_RESID) {
+      for (int m = et256; m < M; m += 256) {
+        float ss = 0.f;
+        for (int t0 = 0; t0 < a.ssq_tiles; t0 += 16) {
+          float p[16];
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            p[k] = t0 + k < a.ssq_tiles ? __ldcg(a.ssq_in + (size_t)(t0 + k) * a.m_cap + m) : 0.f;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) ss += p[k];
+        }
+        rs[m] = 1.0f / sqrtf(ss * a.inv_d + a.eps);
+      }
+      for (int m = M + et256; m < min(M + kEpiTok, kWideMaxRows); m += 256) rs[m] = 0.f;  // the last chunk's other rows
+      all_epi_bar();
+    }
+    auto chunks_of = [&](int w_tile, int tok_base) {
+      return w_tile < a.w_tiles ? max(0, min(n_tok / kEpiTok, (M - tok_base + kEpiTok - 1) / kEpiTok)) : 0;
+    };
+    // A split tile this pair has stored its partial of, and its share of it:
+    // contributor i of n finishes chunks [ceil(i nch / n), ceil((i + 1) nch / n))
+    struct Share {
+      int t, w_tile, tok_base, cf, n, readers, c0, c1;
+    };
+    Share sh0{0, 0, 0, 0, 1, 0, 0, 0}, sh1{0, 0, 0, 0, 1, 0, 0, 0};
+    auto mask_of = [&](int t) { return reinterpret_cast<unsigned long long*>(a.counters) + 2 * t + rank; };
+    auto partial = [&](const Share& h, int k) {
+      // only the tile's first contributor may begin before the tile
+      const int sl = k > 0 || start_of(h.cf) >= h.t * kc ? 0 : 1;
+      return a.partials + ((size_t)(2 * (h.cf + k) + rank) * 2 + sl) * kTileF;
+    };
+    int seg_i = 0, rounds = 0;
+    bool ok = true;
+    int u = u0;
+    // Each turn of the loop takes one segment of this pair's range: a partial
+    // is stored, a whole tile's chunks are finished from the accumulator; and
+    // after the last segment one round of the shares, whose partials a bulk
+    // copy per contributor brings into the ring (idle by then).
+    while (true) {
+      const bool from_acc = u < u1;
+      int take0 = 0, take1 = 0, base1 = 0;  // chunks of this turn: of the tile / first share, of the second share
+      bool staged = true;
+      unsigned long long old0 = 0, old1 = 0;
+      uint32_t tbase = 0;
+      int wt0 = 0, wt1 = 0, tb0 = 0, tb1 = 0, n0 = 0, n1 = 0, ch0 = 0, ch1 = 0;  // tile, token, contributors, first chunk
+      int ab = 0;
+      if (from_acc) {
+        const int t = u / kc;
+        const int ub = u, ue = min((t + 1) * kc, u1);
+        u = ue;
+        ab = seg_i & 1;
+        wt0 = 2 * (t / tok_tiles) + (int)rank;
+        tb0 = t % tok_tiles * n_tok;
+        const int nch = chunks_of(wt0, tb0);
+        const bool whole = ub == t * kc && ue == (t + 1) * kc;
+        if (whole) take0 = nch;
+        ok = mbar_wait(&accf[ab], (uint32_t)((seg_i >> 1) & 1), abort_flag);
+        if (all_epi_any(!ok)) {
+          if (et256 == 0) set_status(a.status, ST_TIMEOUT_EPI);
+          *abort_flag = 1;
+          break;
+        }
+        ++seg_i;
+        tc_fence_after();
+        tbase = tmem + ab * kWideTok + ((uint32_t)(q * 32) << 16);
+        if (!whole) {
+          const int slot = ub == u0 ? 0 : 1;
+          float* mine = a.partials + ((size_t)(2 * c + rank) * 2 + slot) * kTileF;
+#pragma unroll 2
+          for (int ch = grp; ch < nch; ch += 2) {
+            float v[kEpiTok];
+            load_acc(tbase + ch * kEpiTok, v);
+            // [chunk][j4][row] float4s: a warp's stores are 512 contiguous bytes
+            float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kChF) + fr;
+#pragma unroll
+            for (int j4 = 0; j4 < 4; ++j4)
+              dst[j4 * kTileN] = make_float4(v[4 * j4], v[4 * j4 + 1], v[4 * j4 + 2], v[4 * j4 + 3]);
+          }
+          tc_fence_before();
+          all_epi_bar();  // orders every thread's partial before the one release OR
+          if (et == 0) mbar_arrive_remote(&acce[ab], 0);
+          const int cf = owner(t * kc), n = owner((t + 1) * kc - 1) - cf + 1, i = c - cf;
+          if (et256 == 0 && nch > 0) red_release_or64(mask_of(t), 1ull << i);
+          const Share h{t, wt0, tb0, cf, n, min(n, nch), (i * nch + n - 1) / n, ((i + 1) * nch + n - 1) / n};
+          if (slot == 0) sh0 = h;
+          else sh1 = h;
+          continue;
+        }
+      } else {
+        const int rem0 = sh0.c1 - sh0.c0, rem1 = sh1.c1 - sh1.c0;
+        if (rem0 + rem1 == 0) break;
+        n0 = sh0.n; n1 = sh1.n;
+        take0 = min(rem0, kRingChunks / n0);
+        take1 = min(rem1, (kRingChunks - take0 * n0) / n1);
+        staged = take0 + take1 > 0;
+        if (!staged) {  // more contributors than the ring has places: summed from L2
+          take0 = rem0;
+          take1 = rem1;
+        }
+        base1 = take0 * n0;
+        wt0 = sh0.w_tile; tb0 = sh0.tok_base; ch0 = sh0.c0;
+        wt1 = sh1.w_tile; tb1 = sh1.tok_base; ch1 = sh1.c0;
+      }
+      // this group's chunks of the turn: every second of take0 + take1
+      auto tile_of = [&](int i, int& w_tile, int& tok0) {
+        w_tile = i < take0 ? wt0 : wt1;
+        tok0 = i < take0 ? tb0 + (ch0 + i) * kEpiTok : tb1 + (ch1 + i - take0) * kEpiTok;
+      };
+      const int items = take0 + take1;
+      EpiPre pre = {};
+      if (grp < items) {
+        int w_tile, tok0;
+        tile_of(grp, w_tile, tok0);
+        pre = epi_pre<MODE>(a, w_tile, tok0, et, M);
+      }
+      if (!from_acc) {
+        if (et256 == 0) {
+          bool got = true;
+          if (staged) {
+            fence_proxy_async_all();  // the ring was read by the previous round
+            *fx_armed = rounds + 1;
+            mbar_arrive_expect_tx(fx, (uint32_t)(take0 * n0 + take1 * n1) * kChF * 4);
+          }
+          const unsigned long long all0 = take0 ? contrib_bits(n0) : 0, all1 = take1 ? contrib_bits(n1) : 0;
+          unsigned long long seen0 = 0, seen1 = 0;
+          const unsigned long long t0 = globaltimer();
+          // copies of the contributors that have arrived since the last look;
+          // the partials were written through the generic proxy, the copies
+          // read them through the async proxy
+          auto fetch = [&](const Share& h, unsigned long long all, unsigned long long& seen, int take, int at) {
+            const unsigned long long m = ld_acquire_u64(mask_of(h.t)) & all;
+            unsigned long long nw = m & ~seen;
+            if (!nw) return false;
+            fence_proxy_async();
+            while (nw && staged) {
+              const int k = __ffsll((long long)nw) - 1;
+              nw &= nw - 1;
+              bulk_load(reinterpret_cast<float*>(ring) + (size_t)(at + k * take) * kChF, partial(h, k) + (size_t)h.c0 * kChF,
+                        (uint32_t)take * kChF * 4, fx);
+            }
+            seen = m;
+            return true;
+          };
+          while (seen0 != all0 || seen1 != all1) {
+            bool any = false;
+            if (seen0 != all0) any |= fetch(sh0, all0, seen0, take0, 0);
+            if (seen1 != all1) any |= fetch(sh1, all1, seen1, take1, base1);
+            if (!any && (*abort_flag || globaltimer() - t0 > kWaitLimitNs)) {
+              got = false;
+              break;
+            }
+          }
+          if (!got) set_status(a.status, ST_TIMEOUT_EPI);
+          bcast[0] = got ? 1 : 0;
+          // last round of a share: count it in the mask's upper byte (read below)
+          if (got && take0 && sh0.c0 + take0 == sh0.c1)
+            old0 = atomicAdd(mask_of(sh0.t), 1ull << kWideReadShift);
+          if (got && take1 && sh1.c0 + take1 == sh1.c1)
+            old1 = atomicAdd(mask_of(sh1.t), 1ull << kWideReadShift);
+        }
+        all_epi_bar();
+        ok = bcast[0] != 0;
+        if (ok && staged) ok = mbar_wait(fx, (uint32_t)(rounds & 1), abort_flag);
+        if (all_epi_any(!ok)) {
+          if (et256 == 0) set_status(a.status, ST_TIMEOUT_EPI);
+          *abort_flag = 1;
+          break;
+        }
+      }
+#pragma unroll 1
+      for (int i = grp; i < items; i += 2) {
+        const EpiPre now = pre;
+        int w_tile, tok0;
+        if (i + 2 < items) {
+          tile_of(i + 2, w_tile, tok0);
+          pre = epi_pre<MODE>(a, w_tile, tok0, et, M);
+        }
+        tile_of(i, w_tile, tok0);
+        float v[kEpiTok];
+        if (from_acc) {
+          load_acc(tbase + i * kEpiTok, v);
+        } else {
+#pragma unroll
+          for (int j = 0; j < kEpiTok; ++j) v[j] = 0.f;
+          const int n = i < take0 ? n0 : n1, take = i < take0 ? take0 : take1;
+          const int at = i < take0 ? i : base1 + i - take0;
+#pragma unroll 2
+          for (int k = 0; k < n; ++k) {
+            const float4* p;
+            if (staged)
+              p = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(ring) + (size_t)(at + k * take) * kChF) + fr;
+            else
+              p = reinterpret_cast<const float4*>((i < take0 ? partial(sh0, k) : partial(sh1, k)) +
+                                                  (size_t)(i < take0 ? ch0 + i : ch1 + i - take0) * kChF) + fr;
+#pragma unroll
+            for (int j4 = 0; j4 < 4; ++j4) {
+              const float4 pv = staged ? p[j4 * kTileN] : __ldcg(p + j4 * kTileN);
+              v[4 * j4 + 0] += pv.x;
+              v[4 * j4 + 1] += pv.y;
+              v[4 * j4 + 2] += pv.z;
+              v[4 * j4 + 3] += pv.w;
+            }
+          }
+        }
+        epi_chunk<MODE>(a, v, w_tile, tok0, tok0, fr, et, M, S, now);
+      }
+      if (from_acc) {
+        tc_fence_before();
+        epi_bar(S.bar);
+        if (et == 0) mbar_arrive_remote(&acce[ab], 0);
+      } else {
+        if (sh0.c0 + take0 + (sh1.c0 + take1) < sh0.c1 + sh1.c1)
+          all_epi_bar();  // the ring is read out before the next round
+        if (et256 == 0) {
+          // the last of the finishing CTAs clears the mask
+          if (take0 && sh0.c0 + take0 == sh0.c1 && (int)(old0 >> kWideReadShift) == sh0.readers - 1)
+            *mask_of(sh0.t) = 0ull;
+          if (take1 && sh1.c0 + take1 == sh1.c1 && (int)(old1 >> kWideReadShift) == sh1.readers - 1)
+            *mask_of(sh1.t) = 0ull;
+        }
+        sh0.c0 += take0;
+        sh1.c0 += take1;
+        rounds += staged ? 1 : 0;
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (*abort_flag) {
+    // let this CTA's copies and MMAs in flight land before its memory goes away
+    if (warp == 0 && lane == 0)
+      for (int s = 0; s < kWideMaxStages; ++s)
+        if (armed >> s & 1u) mbar_drain(&full[s], (armed_odd >> s & 1u) ^ 1u);
+    if (warp == 1 && rank == 0) {
+      if (elect_one()) umma2_commit(drain, 1);
+      __syncwarp();
+      mbar_drain(drain, 0);
+    }
+    if (threadIdx.x == 64 && *fx_armed) mbar_drain(fx, (uint32_t)((*fx_armed - 1) & 1));
+    __syncthreads();
+  }
+  __syncwarp();
+  cluster_sync();  // the peer's MMAs read this CTA's memory, its threads arrive on this CTA's barriers
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc2(tmem, 512);
+  }
+}
+
+using WideKernel = void (*)(WideArgs);
+static WideKernel wide_kernel(int mode) {
+  switch (mode) {
+    case MODE_QKV: return gemm_wide_kernel<MODE_QKV>;
+    case MODE_RESID: return gemm_wide_kernel<MODE_RESID>;
+    case MODE_SWIGLU: return gemm_wide_kernel<MODE_SWIGLU>;
+    default: return gemm_wide_kernel<MODE_LOGITS>;
+  }
+}
+
+static void wide_launch_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute (&attr)[2], int pairs, cudaStream_t s,
+                               bool pdl) {
+  cfg.gridDim = dim3(2 * pairs);
+  cfg.blockDim = dim3(kWideThreads);
+  cfg.dynamicSmemBytes = kWideSmem;
+  cfg.stream = s;
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 2;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 2 : 1;
+}
+
+int gemm_wide_max_pairs(int sm) {
+  int pairs = sm / 2;
+  for (int mode = 0; mode < 4; ++mode) {
+    cudaError_t e = cudaFuncSetAttribute(wide_kernel(mode), cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSmem);
+    if (e != cudaSuccess) throw e;
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[2];
+    wide_launch_config(cfg, attr, sm / 2, nullptr, false);
+    int n = 0;
+    e = cudaOccupancyMaxActiveClusters(&n, wide_kernel(mode), &cfg);
+    if (e != cudaSuccess) throw e;
+    if (n < pairs) pairs = n;
+  }
+  return pairs < 1 ? 1 : pairs;
+}
+
+void launch_gemm_wide(const WideArgs& a, int pairs, cudaStream_t s, bool pdl) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  wide_launch_config(cfg, attr, pairs, s, pdl);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, wide_kernel(a.g.mode), a);
+  if (e != cudaSuccess) throw e;
+}
+
+}  // namespace pard

@@ -32,10 +32,9 @@ struct CallArgs {
 };
 
 struct GemmArgs {
-  CUtensorMap wmap[kMaxSeg];  // row-major weights (A operand) for shapes that are not packed;
-                              // pair mode: [0] gate, [1] up, 64-row boxes
-  const __nv_bfloat16* wpk[kMaxSeg];  // packed weights (null: use wmap)
-  const __nv_bfloat16* x;     // packed activations (B operand): row 2m = hi(m), 2m+1 = lo(m)
+  CUtensorMap wmap[kMaxSeg];  // weights (A operand), row-major or packed; pair mode: [0] gate, [1] up, 64-row boxes
+  const __nv_bfloat16* wpk[kMaxSeg];  // packed weights (null: wmap is row-major)
+  const __nv_bfloat16* x;     // packed activations (B operand), a hi and a lo row per token (xpk)
   int x_rows;                 // rows of the activation buffer (2 x row capacity)
   int nseg;
   int seg_tile0[kMaxSeg + 1]; // prefix sums of tiles per segment
@@ -223,7 +222,30 @@ constexpr int kMaxGemmTiles = 32768;  // output tiles (weight tile x token tile)
 constexpr int kMaxQVRows = 64;          // query vectors of one attention work unit
 constexpr int kMaxAttnSplit = 16;       // key splits (CTAs of one cluster) of one attention work unit
 
-// launchers (gemm.cu, attention.cu, misc.cu)
+// Wide GEMM (gemm_wide.cu; passes of more than 64 rows): tiles of 256 weight
+// rows and at most kWideTok tokens, multiplied by a pair of CTAs.
+constexpr int kWideTok = 256;
+constexpr int kWideReadShift = 56;  // a split tile's mask word: 56 contributors, and above them its finished shares
+constexpr int kWideMaxRows = 2048;  // rows of one pass (64 sequences x 2 x 16)
+constexpr int kWideBoxL = 32, kWideBoxS = 16;
+struct WideArgs {
+  GemmArgs g;              // packed matrices: wmap holds the packed array as a tensor of 128-byte rows
+  CUtensorMap x[3];        // the activation buffer as one, boxes of g.n_tok, kWideBoxL and kWideBoxS rows
+};
+// Token tiles of a pass of m rows, all of the same size (a multiple of 16).
+__host__ __device__ inline void wide_tiles(int m, int& tiles, int& n_tok) {
+  tiles = (m + kWideTok - 1) / kWideTok;
+  n_tok = ((m + tiles - 1) / tiles + 15) / 16 * 16;
+}
+// Pairs that share U units: at least four units (64 KB of weights a CTA) each,
+// and no more than 56 to a tile of kc units.
+__host__ __device__ inline int wide_pairs(int U, int kc, int max_pairs) {
+  const int least = kc > 4 * 54 ? (kc + 53) / 54 : 4;
+  const int n = U / least;
+  return n < 1 ? 1 : (n < max_pairs ? n : max_pairs);
+}
+
+// launchers (gemm.cu, gemm_wide.cu, attention.cu, misc.cu)
 void launch_embed(const EmbedArgs& a, int grid, cudaStream_t s, bool pdl);
 void launch_gather_rows(const __nv_bfloat16* x, int x_rows, const float* ssq, int ssq_tiles, int m_cap_src, int src_row,
                         __nv_bfloat16* xg, int xg_rows, float* ssqg, int m_cap_dst, int dst_row, int d, cudaStream_t s,
@@ -246,7 +268,8 @@ constexpr int kCodMaxN = 4096;  // rows per subtask of one COD sample
 void launch_cod(int N, int K, double r, double r_min, uint64_t seed, uint64_t sample_id, int32_t* keep,
                 int32_t* counts, cudaStream_t s);
 void launch_gemm(const GemmArgs& a, int tt, int grid, cudaStream_t s, bool pdl);
-int gemm_smem_bytes(int tt);
+int gemm_wide_max_pairs(int sm);  // pairs the GPU holds at once (all of a launch's pairs must be)
+void launch_gemm_wide(const WideArgs& a, int pairs, cudaStream_t s, bool pdl);
 void launch_attention(const AttnArgs& a, int grid_x, cudaStream_t s, bool pdl);
 int attention_rows_per_block(int group);
 

@@ -123,8 +123,8 @@ __global__ void __launch_bounds__(128) embed_kernel(const __grid_constant__ Embe
       a.h[(size_t)m * a.d + c] = h;
       __nv_bfloat16 hi, lo;
       split_bf16(h * __bfloat162float(a.gain0[c]), hi, lo);
-      a.x[xpk(2 * m, c, 2 * a.m_cap)] = hi;
-      a.x[xpk(2 * m + 1, c, 2 * a.m_cap)] = lo;
+      a.x[xpk(m, 0, c, 2 * a.m_cap)] = hi;
+      a.x[xpk(m, 1, c, 2 * a.m_cap)] = lo;
       ss += h * h;
     }
     ss = warp_sum(ss);
@@ -161,8 +161,8 @@ __global__ void gather_rows_kernel(const __nv_bfloat16* x, int x_rows, const flo
   pdl_wait();
   pdl_trigger();
   for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    xg[xpk(2 * dst_row, c, xg_rows)] = x[xpk(2 * src_row, c, x_rows)];
-    xg[xpk(2 * dst_row + 1, c, xg_rows)] = x[xpk(2 * src_row + 1, c, x_rows)];
+    xg[xpk(dst_row, 0, c, xg_rows)] = x[xpk(src_row, 0, c, x_rows)];
+    xg[xpk(dst_row, 1, c, xg_rows)] = x[xpk(src_row, 1, c, x_rows)];
   }
   for (int t = threadIdx.x; t < ssq_tiles; t += blockDim.x)
     ssqg[(size_t)t * m_cap_dst + dst_row] = ssq[(size_t)t * m_cap_src + src_row];

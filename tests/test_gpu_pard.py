@@ -487,3 +487,24 @@ def test_cod_threshold_bins_at_the_edges():
         torch.cuda.synchronize()
         assert counts_g.cpu().tolist() == counts_o, (n, K, r, r_min)
         assert np.array_equal(keep_g.cpu().numpy(), keep_o), (n, K, r, r_min)
+
+
+@pytest.mark.parametrize("batch,K,lens,chunk", [(13, 4, (3, 70), 64), (16, 7, (5, 20), 320), (2, 4, (300, 330), 320),
+                                                (1, 3, (600, 600), 576)],
+                         ids=["65_rows", "128_rows_prefill_odd", "two_token_tiles", "three_token_tiles"])
+def test_wide_gemm_tile_edges(batch, K, lens, chunk):
+    """Passes of more than 64 rows (CTA pairs of 256 weight rows): row counts
+    at and beside a tile's edges, one to three token tiles, odd numbers of
+    128-row weight tiles (d 384, FFN 704, vocabulary 2056: the last pair's
+    second CTA has none), packed and row-major matrices, draft passes with
+    fewer rows than their capacity; two greedy steps against the oracle."""
+    V = 2056
+    shape = S.WORKLOADS["tiny"].target.replace(n_layers=2, d_model=384, ffn=704, vocab=V, mask_id=V - 1)
+    wl = S.WORKLOADS["tiny"].replace(target=shape, draft=shape.replace(n_layers=1, ffn=712), batch=batch, K=K,
+                                     prompt_len=None, prompt_len_range=lens, n_new=12)
+    P = Pair(wl, prefill_chunk=chunk)
+    P.prefill()
+    for step in range(1, 3):
+        greedy_step(P, step)
+    assert P.eng.last_status() == 0
+    print("stats", P.stats)
