@@ -449,7 +449,7 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int batch
     a.page_size = c->lim.page_size; a.n_pages = c->lim.n_pages;
     a.row_blocks = geo.row_blocks; a.n_split = geo.n_split;
     a.nbuf = geo.nbuf;
-    a.scale = (float)(1.0 / std::sqrt((double)cf.head_dim));
+    a.scale = (float)(1.4426950408889634 / std::sqrt((double)cf.head_dim));  // scores in units of log 2
     a.x_out = c->xo; a.x_rows = 2 * c->D.MC;
     a.status = c->status;
     a.paths = c->paths;

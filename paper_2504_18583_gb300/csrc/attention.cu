@@ -26,7 +26,8 @@ namespace pard {
 // than twice over (ragged batches with long contexts), where the latency of
 // a unit's dependent steps is hidden by the other CTAs' warps instead.
 template <int HD, int GROUP, int NBUF>
-__global__ void __launch_bounds__(kAttnThreads) attn_kernel(const __grid_constant__ AttnArgs a) {
+__global__ void __launch_bounds__(kAttnThreads, NBUF == 2 ? (HD == 64 ? 5 : 4) : (HD == 64 ? 4 : 2))
+    attn_kernel(const __grid_constant__ AttnArgs a) {
   using C = AttnCfg<HD, NBUF>;
   constexpr int LD = C::kPartLd;
   extern __shared__ __align__(128) uint8_t smem[];
@@ -116,7 +117,7 @@ __global__ void __launch_bounds__(kAttnThreads) attn_kernel(const __grid_constan
         float mx = m;
 #pragma unroll
         for (int off = 8; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off, 16));
-        const float w = m == -INFINITY ? 0.f : expf(m - mx);
+        const float w = m == -INFINITY ? 0.f : exp2_fast(m - mx);
         float L = live ? recv[((size_t)sr * cnt + r) * LD + HD + 1] * w : 0.f;
 #pragma unroll
         for (int off = 8; off > 0; off >>= 1) L += __shfl_xor_sync(0xffffffffu, L, off, 16);
@@ -144,42 +145,41 @@ __global__ void __launch_bounds__(kAttnThreads) attn_kernel(const __grid_constan
     return;
   }
   cluster_sync();
-  // Pull combine, in rank order; CTA `rank` finishes query vectors rank,
-  // rank+NS, ...  Each thread takes one output pair (qv, d..d+1) at a time
-  // and requests every rank's (max, sum) and partial values before using any,
-  // so a round of work is one distributed-shared-memory round trip.
-  const int my_qv = nqv > (int)rank ? (nqv - (int)rank + (int)NS - 1) / (int)NS : 0;
-  const int n_items = my_qv * (HD / 2);
-  for (int i = threadIdx.x; i < n_items; i += kAttnThreads) {
-    const int qv = (int)rank + (int)NS * (i / (HD / 2)), d = 2 * (i % (HD / 2));
-    float2 ml[kMaxCluster], pv[kMaxCluster];
+  // Pull combine, in rank order; CTA `rank` finishes query vectors
+  // [rank cnt, (rank + 1) cnt).  A thread takes four columns of a row and
+  // requests every rank's (max, sum) and piece before using any: one
+  // distributed-shared-memory round trip for 128 pieces.  (Two columns a
+  // thread took 9k clocks at 9 splits, the weights in a round trip of their
+  // own 5.7k.)
+  const int my0 = (int)rank * cnt;
+  const int my_n = max(0, min(nqv, my0 + cnt) - my0);
+  for (int i = threadIdx.x; i < my_n * (HD / 4); i += kAttnThreads) {
+    const int qv = my0 + i / (HD / 4), d4 = i % (HD / 4);
+    const float* row = part + (size_t)qv * LD;
+    float2 ml[kMaxCluster];
+    float4 v[kMaxCluster];
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r) {
       const bool live = r < (int)NS;
-      ml[r] = live ? ld_dsmem2(part + qv * LD + HD, (uint32_t)r) : make_float2(-INFINITY, 0.f);
-      pv[r] = live ? ld_dsmem2(part + qv * LD + d, (uint32_t)r) : make_float2(0.f, 0.f);
+      ml[r] = live ? ld_dsmem2(row + HD, (uint32_t)r) : make_float2(-INFINITY, 0.f);
+      v[r] = live ? ld_dsmem4(row + 4 * d4, (uint32_t)r) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
     float mx = -INFINITY;
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r) mx = fmaxf(mx, ml[r].x);
     float L = 0.f;
-    float2 acc = make_float2(0.f, 0.f);
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int r = 0; r < kMaxCluster; ++r) {
-      const float w = ml[r].x == -INFINITY ? 0.f : expf(ml[r].x - mx);
+      const float w = ml[r].x == -INFINITY ? 0.f : exp2_fast(ml[r].x - mx);
       L += ml[r].y * w;
-      acc.x += pv[r].x * w;
-      acc.y += pv[r].y * w;
+      acc.x += v[r].x * w;
+      acc.y += v[r].y * w;
+      acc.z += v[r].z * w;
+      acc.w += v[r].w * w;
     }
-    const int m = row0 + qv / GROUP;
-    const int col = (kvh * GROUP + qv % GROUP) * HD + d;
-    __nv_bfloat16 h0, l0, h1, l1;
-    split_bf16(acc.x / L, h0, l0);
-    split_bf16(acc.y / L, h1, l1);
-    *reinterpret_cast<uint32_t*>(a.x_out + xpk(m, 0, col, a.x_rows)) =
-        (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    *reinterpret_cast<uint32_t*>(a.x_out + xpk(m, 1, col, a.x_rows)) =
-        (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+    store_pair4(a.x_out, row0 + qv / GROUP, (kvh * GROUP + qv % GROUP) * HD + 4 * d4, a.x_rows,
+                make_float4(acc.x / L, acc.y / L, acc.z / L, acc.w / L));
   }
   cluster_sync();  // peers may still be reading this CTA's partial
 }

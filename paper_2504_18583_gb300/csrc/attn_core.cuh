@@ -14,6 +14,7 @@ constexpr int kAttnThreads = 128;  // 4 warps x 16 query vectors
 constexpr int kMaxQV = kMaxQVRows;
 constexpr int kKeyChunk = 32;
 constexpr int kMaxCluster = kMaxAttnSplit;  // key splits of one work unit (clusters above 8 are non-portable)
+constexpr int kAttnPage = 16;         // tokens of a KV page (the only size the library takes)
 constexpr int kAttnPageCache = 512;  // page ids of one work unit's key range held in shared memory
 
 // Shared memory of one work unit: NBUF K/V chunk buffers (a ring, NBUF - 1
@@ -33,8 +34,9 @@ struct AttnCfg {
   static constexpr int kSmem = kPageOff + kAttnPageCache * 4 + 256;
 };
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+// 16 bytes, or 16 zero bytes without reading src
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool read) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(read ? 16 : 0) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
@@ -61,15 +63,29 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(addr));
 }
-__device__ __forceinline__ void ldsm_x2_trans(uint32_t& r0, uint32_t& r1, uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
 }
-// two consecutive floats (8-byte aligned) of CTA `rank`'s shared memory
+// 2^x (2 ulp; exactly 0 at -infinity)
+__device__ __forceinline__ float exp2_fast(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+// two or four consecutive floats (8- or 16-byte aligned) of CTA `rank`'s shared memory
 __device__ __forceinline__ float2 ld_dsmem2(const float* local, uint32_t rank) {
-  uint32_t remote;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(local)), "r"(rank));
   float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(remote) : "memory");
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(mapa_shared(local, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_dsmem4(const float* local, uint32_t rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(mapa_shared(local, rank))
+               : "memory");
   return v;
 }
 
@@ -96,33 +112,41 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 
 // K and V rows of one 32-key chunk into shared memory; positions past maxpos
 // (masked anyway) and bad pages become zeros.  spg: the sequence's page table
-// row in shared memory (nullptr: read it from global memory here).
+// row in shared memory (nullptr: read it from global memory here).  A chunk
+// is two pages of 16 tokens: a thread's row within a page is the same for
+// every piece (two with hd = 128), so a piece costs one add per tensor.
+// (With the page size read at run time, two divisions and a page lookup a
+// piece took 2.3k clocks a chunk, more than the chunk's MMAs.)
 template <int HD, int NBUF>
 __device__ __forceinline__ void load_chunk(const AttnArgs& a, const int* pt, const int* spg, int kvh, int chunk,
                                            int maxpos, uint8_t* sK, uint8_t* sV, int tid) {
   using C = AttnCfg<HD, NBUF>;
-  constexpr int kCh = HD * 2 / 16;
-  for (int i = tid; i < kKeyChunk * kCh; i += kAttnThreads) {
-    const int key = i / kCh, ch = i % kCh;
-    const int pos = chunk * kKeyChunk + key;
-    uint8_t* dk = sK + key * C::kRowBytes + ch * 16;
-    uint8_t* dv = sV + key * C::kRowBytes + ch * 16;
+  constexpr int kCh = HD * 2 / 16;               // 16-byte pieces a row
+  constexpr int kRows = kAttnThreads / kCh;      // rows a sweep of the threads covers: 8 or 16
+  constexpr int kSweeps = kAttnPage / kRows;     // sweeps a page
+  const int ch = tid % kCh, row0 = tid / kCh;
+  const size_t page_elems = (size_t)a.hkv * kAttnPage * HD;
+  const size_t in_page = ((size_t)kvh * kAttnPage + row0) * HD + ch * 8;
+  const uint32_t dk = smem_u32(sK) + row0 * C::kRowBytes + ch * 16, dv = smem_u32(sV) + row0 * C::kRowBytes + ch * 16;
+#pragma unroll
+  for (int h = 0; h < kKeyChunk / kAttnPage; ++h) {
+    const int pi = chunk * (kKeyChunk / kAttnPage) + h;  // page index within the sequence
     int page = -1;
-    if (pos <= maxpos && pos / a.page_size < a.pt_ld) {
-      page = spg ? spg[pos / a.page_size] : pt[pos / a.page_size];
+    if (pi * kAttnPage <= maxpos && pi < a.pt_ld) {
+      page = spg ? spg[pi] : pt[pi];
       if (page < 0 || page >= a.n_pages) {
         set_status(a.status, ST_BAD_PAGE);
         page = -1;
       }
     }
-    if (page < 0) {
-      *reinterpret_cast<uint4*>(dk) = make_uint4(0, 0, 0, 0);
-      *reinterpret_cast<uint4*>(dv) = make_uint4(0, 0, 0, 0);
-      continue;
+    const size_t off = (size_t)max(page, 0) * page_elems + in_page;
+#pragma unroll
+    for (int w = 0; w < kSweeps; ++w) {
+      const int r = h * kAttnPage + w * kRows;
+      const bool read = page >= 0 && chunk * kKeyChunk + r + row0 <= maxpos;
+      cp_async16(dk + r * C::kRowBytes, a.kcache + off + (size_t)w * kRows * HD, read);
+      cp_async16(dv + r * C::kRowBytes, a.vcache + off + (size_t)w * kRows * HD, read);
     }
-    const size_t off = (((size_t)page * a.hkv + kvh) * a.page_size + pos % a.page_size) * HD + ch * 8;
-    cp_async16(dk, a.kcache + off);
-    cp_async16(dv, a.vcache + off);
   }
 }
 
@@ -163,13 +187,17 @@ constexpr int kKeyHalvesMinChunks = 3;
 // of the chunk ch landed in sK / sV (fp16): S = Q K^T on NJG 8-key n-tiles,
 // scale and causal mask (key position <= row position), running max / sum
 // update with the rescale of o, then O += P V with P as the A fragments.
+// Scores and maxima are in units of log 2 (scale holds the factor), so that a
+// probability is one ex2.
 template <int HD, int NJG, int ROWB>
 __device__ __forceinline__ void attn_chunk(const uint8_t* sK, const uint8_t* sV, int koff, int ch, uint32_t q_base,
                                            int posa, int posb, float scale, float (&o)[HD / 8][4], float& ma,
                                            float& mb, float& la, float& lb, int lane) {
   constexpr int KS = HD / 16;
   constexpr int NT = HD / 8;
-  const int g = lane >> 2, c4 = lane & 3;
+  const int c4 = lane & 3;
+  // ldmatrix.x4 row address of this lane: two n-tiles of 8 keys, both 8-column halves of a k-step
+  const uint32_t k_base = smem_u32(sK + (koff + ((lane >> 4) & 1) * 8 + (lane & 7)) * ROWB) + ((lane >> 3) & 1) * 16;
   // NACC accumulator sets over alternate k-steps keep four independent MMA
   // chains in flight when the warp covers only NJG = 2 n-tiles
   constexpr int NACC = NJG >= 4 ? 1 : 4 / NJG;
@@ -180,17 +208,13 @@ __device__ __forceinline__ void attn_chunk(const uint8_t* sK, const uint8_t* sV,
     for (int j = 0; j < NJG; ++j) sacc[r][j][0] = sacc[r][j][1] = sacc[r][j][2] = sacc[r][j][3] = 0.f;
 #pragma unroll
   for (int ks = 0; ks < KS; ++ks) {
-    uint32_t qf[4], kb[NJG][2];
+    uint32_t qf[4], kb[NJG / 2][4];
     ldsm_x4(qf, q_base + ks * 32);
 #pragma unroll
-    for (int j = 0; j < NJG; ++j) {
-      const uint8_t* krow = sK + (koff + j * 8 + g) * ROWB;
-      kb[j][0] = *reinterpret_cast<const uint32_t*>(krow + (ks * 16 + 2 * c4) * 2);
-      kb[j][1] = *reinterpret_cast<const uint32_t*>(krow + (ks * 16 + 8 + 2 * c4) * 2);
-    }
+    for (int j = 0; j < NJG / 2; ++j) ldsm_x4(kb[j], k_base + j * 16 * ROWB + ks * 32);
     // independent accumulators back to back
 #pragma unroll
-    for (int j = 0; j < NJG; ++j) mma_f16_16816(sacc[ks % NACC][j], qf, kb[j][0], kb[j][1]);
+    for (int j = 0; j < NJG; ++j) mma_f16_16816(sacc[ks % NACC][j], qf, kb[j >> 1][(j & 1) * 2], kb[j >> 1][(j & 1) * 2 + 1]);
   }
   float s[NJG][4];
 #pragma unroll
@@ -219,15 +243,15 @@ __device__ __forceinline__ void attn_chunk(const uint8_t* sK, const uint8_t* sV,
   mxb = fmaxf(mxb, __shfl_xor_sync(0xffffffffu, mxb, 1));
   mxb = fmaxf(mxb, __shfl_xor_sync(0xffffffffu, mxb, 2));
   const float mna = fmaxf(ma, mxa), mnb = fmaxf(mb, mxb);
-  const float ca = mna == -INFINITY ? 1.f : expf(ma - mna);
-  const float cb = mnb == -INFINITY ? 1.f : expf(mb - mnb);
+  const float ca = mna == -INFINITY ? 1.f : exp2_fast(ma - mna);
+  const float cb = mnb == -INFINITY ? 1.f : exp2_fast(mb - mnb);
   float sa = 0.f, sb = 0.f;
 #pragma unroll
   for (int j = 0; j < NJG; ++j) {
-    s[j][0] = s[j][0] == -INFINITY ? 0.f : expf(s[j][0] - mna);
-    s[j][1] = s[j][1] == -INFINITY ? 0.f : expf(s[j][1] - mna);
-    s[j][2] = s[j][2] == -INFINITY ? 0.f : expf(s[j][2] - mnb);
-    s[j][3] = s[j][3] == -INFINITY ? 0.f : expf(s[j][3] - mnb);
+    s[j][0] = s[j][0] == -INFINITY ? 0.f : exp2_fast(s[j][0] - mna);
+    s[j][1] = s[j][1] == -INFINITY ? 0.f : exp2_fast(s[j][1] - mna);
+    s[j][2] = s[j][2] == -INFINITY ? 0.f : exp2_fast(s[j][2] - mnb);
+    s[j][3] = s[j][3] == -INFINITY ? 0.f : exp2_fast(s[j][3] - mnb);
     sa += s[j][0] + s[j][1];
     sb += s[j][2] + s[j][3];
   }
@@ -251,14 +275,14 @@ __device__ __forceinline__ void attn_chunk(const uint8_t* sK, const uint8_t* sV,
     pf[1] = pack_h2(s[2 * kk][2], s[2 * kk][3]);
     pf[2] = pack_h2(s[2 * kk + 1][0], s[2 * kk + 1][1]);
     pf[3] = pack_h2(s[2 * kk + 1][2], s[2 * kk + 1][3]);
-    const uint32_t vrow = smem_u32(sV + (koff + kk * 16 + (lane & 15)) * ROWB);
+    const uint32_t vrow = smem_u32(sV + (koff + kk * 16 + (lane & 15)) * ROWB) + (lane >> 4) * 16;
 #pragma unroll
     for (int n0 = 0; n0 < NT; n0 += 4) {
-      uint32_t vb[4][2];
+      uint32_t vb[2][4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) ldsm_x2_trans(vb[u][0], vb[u][1], vrow + (n0 + u) * 16);
+      for (int u = 0; u < 2; ++u) ldsm_x4_trans(vb[u], vrow + (n0 + 2 * u) * 16);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) mma_f16_16816(o[n0 + u], pf, vb[u][0], vb[u][1]);
+      for (int u = 0; u < 4; ++u) mma_f16_16816(o[n0 + u], pf, vb[u >> 1][(u & 1) * 2], vb[u >> 1][(u & 1) * 2 + 1]);
     }
   }
 }
@@ -347,8 +371,9 @@ __device__ AttnRows attn_unit(const AttnArgs& a, int b, int kvh, int rb, int sp,
   // q is rewritten by every layer (by the previous kernel): L2 loads
   constexpr int kQIter = kMaxQV * (HD / 4) / kAttnThreads;  // 8 or 16 float4 per thread
   constexpr int kQGroup = kQIter < 8 ? kQIter : 8;
+  const int q_sweeps = min(kQIter, ((nqv + 15) / 16 * 16 * (HD / 4) + kAttnThreads - 1) / kAttnThreads);  // whole 16-row tiles
 #pragma unroll 1
-  for (int i0 = 0; i0 < kQIter; i0 += kQGroup) {
+  for (int i0 = 0; i0 < q_sweeps; i0 += kQGroup) {
     float4 v[kQGroup];
 #pragma unroll
     for (int u = 0; u < kQGroup; ++u) {
@@ -450,8 +475,8 @@ __device__ AttnRows attn_unit(const AttnArgs& a, int b, int kvh, int rb, int sp,
       const float2 mla = *reinterpret_cast<const float2*>(twin + qa * C::kPartLd + HD);
       const float2 mlb = *reinterpret_cast<const float2*>(twin + qb * C::kPartLd + HD);
       const float na = fmaxf(ma, mla.x), nb = fmaxf(mb, mlb.x);
-      const float sa0 = ma == -INFINITY ? 0.f : expf(ma - na), sa1 = mla.x == -INFINITY ? 0.f : expf(mla.x - na);
-      const float sb0 = mb == -INFINITY ? 0.f : expf(mb - nb), sb1 = mlb.x == -INFINITY ? 0.f : expf(mlb.x - nb);
+      const float sa0 = ma == -INFINITY ? 0.f : exp2_fast(ma - na), sa1 = mla.x == -INFINITY ? 0.f : exp2_fast(mla.x - na);
+      const float sb0 = mb == -INFINITY ? 0.f : exp2_fast(mb - nb), sb1 = mlb.x == -INFINITY ? 0.f : exp2_fast(mlb.x - nb);
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
         const int d = nt * 8 + 2 * c4;
