@@ -99,8 +99,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
     u0 = range_start(c, U, G);
     u1 = range_start(c + 1, U, G);
   }
-  uint32_t armed[C::kStages];  // producer: times each ring slot was armed
-  for (int s = 0; s < C::kStages; ++s) armed[s] = 0;
+  uint32_t armed = 0, armed_odd = 0;  // producer: slots armed at least once, and those armed an odd number of times
   // ring slots this launch uses, and how many are filled before the PDL wait
   const int R = (a.stages > 0 && a.stages < C::kStages) ? a.stages : C::kStages;
   const int P = (a.pre_stages > 0 && a.pre_stages < R) ? a.pre_stages : R;
@@ -112,10 +111,10 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
-    if (lane == 0) {
+    // The whole warp runs the loop and one elected thread issues: inside "if
+    // (lane == 0)" every copy (and every MMA below) takes about 100 clocks to issue.
+    {
       const uint64_t pol = policy_evict_first();
-      for (int i = 0; i < kMaxSeg; ++i)
-        if ((i < a.nseg || (a.pair && i < 2)) && !a.wpk[i]) tma_prefetch_desc(&a.wmap[i]);
       const int n = u1 - u0;
       const int npre = n < P ? n : P;
       // Unit cursor advanced incrementally: the producer issues one stage per
@@ -174,37 +173,49 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
         }
       };
       // weights first: they do not depend on the previous kernel
-      int pre_kk[C::kStages], pre_tok[C::kStages];
+      auto arm = [&](int s) {
+        armed |= 1u << s;
+        armed_odd ^= 1u << s;
+      };
+      const int kk0 = kk, tok0 = tok_tile;
       for (int i = 0; i < npre; ++i) {
-        mbar_arrive_expect_tx(&full[i], stage_bytes);
-        ++armed[i];
-        issue_a(i);
-        pre_kk[i] = kk;
-        pre_tok[i] = tok_tile;
+        arm(i);
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&full[i], stage_bytes);
+          issue_a(i);
+        }
+        __syncwarp();
         advance();
       }
       pdl_wait();
-      for (int i = 0; i < npre; ++i) issue_b(i, pre_kk[i], pre_tok[i]);
+      for (int i = 0, k2 = kk0, t2 = tok0; i < npre; ++i) {
+        if (elect_one()) issue_b(i, k2, t2);
+        __syncwarp();
+        if (++k2 == a.kc) { k2 = 0; if (++t2 == tok_tiles) t2 = 0; }
+      }
       int s = npre % R;
       uint32_t ph = (uint32_t)((npre / R) & 1) ^ 1u;
       for (int i = npre; i < n; ++i) {
-        if (!mbar_wait(&empty[s], ph, abort_flag)) {
-          set_status(a.status, ST_TIMEOUT_TMA);
+        if (!__all_sync(0xffffffffu, mbar_wait(&empty[s], ph, abort_flag))) {
+          if (lane == 0) set_status(a.status, ST_TIMEOUT_TMA);
           *abort_flag = 1;
           break;
         }
-        mbar_arrive_expect_tx(&full[s], stage_bytes);
-        ++armed[s];
-        issue_a(s);
-        issue_b(s, kk, tok_tile);
+        arm(s);
+        if (elect_one()) {
+          mbar_arrive_expect_tx(&full[s], stage_bytes);
+          issue_a(s);
+          issue_b(s, kk, tok_tile);
+        }
+        __syncwarp();
         advance();
         if (++s == R) { s = 0; ph ^= 1u; }
       }
-      pdl_trigger();
+      if (lane == 0) pdl_trigger();
     }
   } else if (warp == 1) {
     // ---------------- MMA issuer ----------------
-    if (lane == 0) {
+    {
       const uint32_t idesc = idesc_bf16(kTileN, 2 * n_tok);
       int s = 0;          // ring slot of the next unit
       uint32_t fph = 0;   // its 'full' phase parity
@@ -215,25 +226,29 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
         const int ub = u, ue = (t + 1) * a.kc < u1 ? (t + 1) * a.kc : u1;
         const int ab = seg_i % C::kNumAcc;
         const uint32_t aph = (uint32_t)((seg_i / C::kNumAcc) & 1) ^ 1u;
-        if (!mbar_wait(&acce[ab], aph, abort_flag)) { ok = false; break; }
+        ok = __all_sync(0xffffffffu, mbar_wait(&acce[ab], aph, abort_flag));
+        if (!ok) break;
         tc_fence_after();
         const uint32_t d = tmem + ab * C::kAccCols;
         for (; u < ue; ++u) {
-          if (!mbar_wait(&full[s], fph, abort_flag)) { ok = false; break; }
+          ok = __all_sync(0xffffffffu, mbar_wait(&full[s], fph, abort_flag));
+          if (!ok) break;
           tc_fence_after();
           const uint64_t ad = sw128_desc(smem_u32(sA + s * C::kABytes));
           const uint64_t bd = sw128_desc(smem_u32(sB + s * C::kBBytes));
+          if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kChunkK / 16; ++k)
-            umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (u > ub || k > 0) ? 1u : 0u);
-          umma_commit(&empty[s]);
+            for (int k = 0; k < kChunkK / 16; ++k)
+              umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (u > ub || k > 0) ? 1u : 0u);
+            umma_commit(&empty[s]);
+            if (u + 1 == ue) umma_commit(&accf[ab]);
+          }
+          __syncwarp();
           if (++s == R) { s = 0; fph ^= 1u; }
         }
-        if (!ok) break;
-        umma_commit(&accf[ab]);
         ++seg_i;
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         set_status(a.status, ST_TIMEOUT_MMA);
         *abort_flag = 1;
       }
@@ -291,9 +306,10 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
     // let this CTA's copies and MMAs in flight land before its memory goes away
     if (warp == 0 && lane == 0)
       for (int s = 0; s < C::kStages; ++s)
-        if (armed[s]) mbar_drain(&full[s], (armed[s] - 1) & 1u);
-    if (warp == 1 && lane == 0) {
-      umma_commit(drain);
+        if (armed >> s & 1u) mbar_drain(&full[s], (armed_odd >> s & 1u) ^ 1u);
+    if (warp == 1) {
+      if (elect_one()) umma_commit(drain);
+      __syncwarp();
       mbar_drain(drain, 0);
     }
     // fx_armed: 1 + the staging round whose copies may be in flight
