@@ -304,9 +304,12 @@ struct pard_ctx {
 
 namespace {
 
+CallArgs call_of(pard_ctx* c, uint64_t seed, uint64_t step, float temp, int sample) {
+  return CallArgs{seed, step, temp, sample, c->K, 0};
+}
+
 void set_call(pard_ctx* c, uint64_t seed, uint64_t step, float temp, int sample, cudaStream_t s) {
-  CallArgs v{seed, step, temp, sample, c->K, 0};
-  launch_set_call(c->call, v, s, true);
+  launch_set_call(c->call, call_of(c, seed, step, temp, sample), s, true);
   c->launches++;
 }
 
@@ -527,7 +530,7 @@ void run_layers(pard_ctx* c, int mi, int rows_cap, int batch, int rows_per_seq, 
 
 // LM head over the packed activation rows x (final-norm scale from ssq_in).
 GemmArgs lm_args(pard_ctx* c, int mi, const __nv_bfloat16* x, int x_rows, const float* ssq_in, int rows_cap, int tt,
-                 const int* m_dev, float* logits, const int* row_out, const int* row_gi, const int* row_seq,
+                 const int* m_dev, float* logits, float* logits_out, const int* row_out, const int* row_gi, const int* row_seq,
                  float4* stats, int2* stats_i, int gumbel_stream) {
   Model& M = c->m[mi];
   GemmArgs a = gemm_base(c, rows_cap, tt);
@@ -541,17 +544,17 @@ GemmArgs lm_args(pard_ctx* c, int mi, const __nv_bfloat16* x, int x_rows, const 
   a.kc = (M.cfg.d_model + kChunkK - 1) / kChunkK;
   a.mode = MODE_LOGITS;
   a.ssq_in = ssq_in; a.ssq_tiles = M.cfg.d_model / 128; a.inv_d = 1.0f / M.cfg.d_model; a.eps = M.cfg.rms_eps;
-  a.logits = logits; a.row_out = row_out; a.row_gi = row_gi; a.row_seq = row_seq;
+  a.logits = logits; a.logits_out = logits_out; a.row_out = row_out; a.row_gi = row_gi; a.row_seq = row_seq;
   a.stats = stats; a.stats_i = stats_i; a.vocab = M.cfg.vocab; a.gumbel_stream = gumbel_stream;
   a.m_early = 1;  // the LM head follows the whole layer stack (or the prefill's gather), far from its row count's writer
   return a;
 }
 
 void run_lm_head(pard_ctx* c, int mi, const __nv_bfloat16* x, int x_rows, const float* ssq_in, int rows_cap, int tt,
-                 const int* m_dev, float* logits, const int* row_out, const int* row_gi, const int* row_seq,
+                 const int* m_dev, float* logits, float* logits_out, const int* row_out, const int* row_gi, const int* row_seq,
                  float4* stats, int2* stats_i, int gumbel_stream, cudaStream_t s) {
-  GemmArgs a = lm_args(c, mi, x, x_rows, ssq_in, rows_cap, tt, m_dev, logits, row_out, row_gi, row_seq, stats, stats_i,
-                       gumbel_stream);
+  GemmArgs a = lm_args(c, mi, x, x_rows, ssq_in, rows_cap, tt, m_dev, logits, logits_out, row_out, row_gi, row_seq, stats,
+                       stats_i, gumbel_stream);
   run_gemm(c, a, tt, s);
 }
 
@@ -876,7 +879,7 @@ pard_status pard_prefill(pard_ctx* c, const int32_t* d_tokens, const int32_t* h_
       offset += len;
     }
     const int gtt = pick_tt(c->D.gcap);
-    run_lm_head(c, 0, c->xg, 2 * c->D.gcap, c->ssqg, batch, gtt, c->g_m, nullptr, nullptr, sample ? c->g_row_gi : nullptr,
+    run_lm_head(c, 0, c->xg, 2 * c->D.gcap, c->ssqg, batch, gtt, c->g_m, nullptr, nullptr, nullptr, sample ? c->g_row_gi : nullptr,
                 c->g_row_seq, c->stats_t, c->stats_it, STREAM_BONUS, s);
     SelectArgs sa;
     std::memset(&sa, 0, sizeof(sa));
@@ -904,16 +907,17 @@ pard_status pard_draft(pard_ctx* c, int32_t sample, float temperature, uint64_t 
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   c->launches = 0;
   return guarded([&]() -> pard_status {
-    set_call(c, seed, step, temperature > 0.f ? temperature : 1.0f, sample, s);
     const int rows_cap = c->batch * 2 * c->K;
     EmbedArgs e = embed_base(c, 1, EMB_DRAFT);
+    e.call = call_of(c, seed, step, temperature > 0.f ? temperature : 1.0f, sample);
+    e.call_out = c->call;
     launch_embed(e, rows_cap, s, true);
     c->launches++;
     Model& M = c->m[1];
     const int keep = (sample || d_logits) ? 1 : 0;
     run_layers(c, 1, rows_cap, c->batch, 2 * c->K, M.page_table, s);
     run_lm_head(c, 1, c->xd, 2 * c->D.MC, c->ssq, rows_cap, pick_tt(rows_cap), c->rp.m_dev,
-                keep ? c->dlogits : nullptr, c->rp.row_out, c->rp.row_gi, c->rp.row_seq, c->stats_d, c->stats_id,
+                keep ? c->dlogits : nullptr, d_logits, c->rp.row_out, c->rp.row_gi, c->rp.row_seq, c->stats_d, c->stats_id,
                 STREAM_DRAFT, s);
     SelectArgs sa;
     std::memset(&sa, 0, sizeof(sa));
@@ -923,8 +927,6 @@ pard_status pard_draft(pard_ctx* c, int32_t sample, float temperature, uint64_t 
     sa.seq_row0 = c->rp.seq_row0; sa.out = d_out;
     launch_select(sa, s, true);
     c->launches++;
-    if (d_logits)
-      CK(cudaMemcpyAsync(d_logits, c->dlogits, (size_t)c->batch * c->K * c->D.vocab * 4, cudaMemcpyDeviceToDevice, s));
     c->last_draft_sampled = sample != 0;
     return PARD_OK;
   });
@@ -942,7 +944,6 @@ pard_status pard_draft_sequential(pard_ctx* c, int32_t sample, float temperature
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   c->launches = 0;
   return guarded([&]() -> pard_status {
-    set_call(c, seed, step, temperature > 0.f ? temperature : 1.0f, sample, s);
     Model& M = c->m[1];
     const int keep = (sample || d_logits) ? 1 : 0;
     for (int i = 0; i < c->K; ++i) {
@@ -951,11 +952,13 @@ pard_status pard_draft_sequential(pard_ctx* c, int32_t sample, float temperature
       const int rows_cap = c->batch * per_seq;
       EmbedArgs e = embed_base(c, 1, EMB_DRAFT_SEQ);
       e.seq_i = i;
+      e.call = call_of(c, seed, step, temperature > 0.f ? temperature : 1.0f, sample);
+      e.call_out = c->call;
       launch_embed(e, rows_cap, s, true);
       c->launches++;
       run_layers(c, 1, rows_cap, c->batch, per_seq, M.page_table, s);
       run_lm_head(c, 1, c->xd, 2 * c->D.MC, c->ssq, rows_cap, pick_tt(rows_cap), c->rp.m_dev,
-                  keep ? c->dlogits : nullptr, c->rp.row_out, c->rp.row_gi, c->rp.row_seq, c->stats_d, c->stats_id,
+                  keep ? c->dlogits : nullptr, d_logits, c->rp.row_out, c->rp.row_gi, c->rp.row_seq, c->stats_d, c->stats_id,
                   STREAM_DRAFT, s);
       SelectArgs sa;
       std::memset(&sa, 0, sizeof(sa));
@@ -967,8 +970,6 @@ pard_status pard_draft_sequential(pard_ctx* c, int32_t sample, float temperature
       launch_select(sa, s, true);
       c->launches++;
     }
-    if (d_logits)
-      CK(cudaMemcpyAsync(d_logits, c->dlogits, (size_t)c->batch * c->K * c->D.vocab * 4, cudaMemcpyDeviceToDevice, s));
     c->last_draft_sampled = sample != 0;
     return PARD_OK;
   });
@@ -981,9 +982,10 @@ pard_status pard_verify(pard_ctx* c, const int32_t* d_draft_in, float temperatur
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   c->launches = 0;
   return guarded([&]() -> pard_status {
-    set_call(c, 0, 0, temperature > 0.f ? temperature : 1.0f, c->last_draft_sampled ? 1 : 0, s);
     const int rows_cap = c->batch * (c->K + 1);
     EmbedArgs e = embed_base(c, 0, EMB_VERIFY);
+    e.call = call_of(c, 0, 0, temperature > 0.f ? temperature : 1.0f, c->last_draft_sampled ? 1 : 0);
+    e.call_out = c->call;
     e.d_in = d_draft_in ? d_draft_in : c->st.d;
     if (!d_draft_in && c->st.kmax != c->K) {
       // internal candidates have row pitch kmax; feed them through a packed copy
@@ -998,11 +1000,8 @@ pard_status pard_verify(pard_ctx* c, const int32_t* d_draft_in, float temperatur
     const int keep = (c->last_draft_sampled || d_logits_out || c->K == 0) ? 1 : 0;
     run_layers(c, 0, rows_cap, c->batch, c->K + 1, M.page_table, s, c->K + 1);  // K + 1 rows per sequence
     run_lm_head(c, 0, c->xd, 2 * c->D.MC, c->ssq, rows_cap, pick_tt(rows_cap), c->rp.m_dev,
-                keep ? c->logits : nullptr, c->rp.row_out, nullptr, c->rp.row_seq, c->stats_t, c->stats_it,
+                keep ? c->logits : nullptr, d_logits_out, c->rp.row_out, nullptr, c->rp.row_seq, c->stats_t, c->stats_it,
                 STREAM_BONUS, s);
-    if (d_logits_out)
-      CK(cudaMemcpyAsync(d_logits_out, c->logits, (size_t)c->batch * (c->K + 1) * c->D.vocab * 4,
-                         cudaMemcpyDeviceToDevice, s));
     return PARD_OK;
   });
 }
@@ -1016,12 +1015,11 @@ pard_status pard_accept_commit(pard_ctx* c, int32_t sample, float temperature, u
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   c->launches = 0;
   return guarded([&]() -> pard_status {
-    set_call(c, seed, step, temperature > 0.f ? temperature : 1.0f, sample, s);
     AcceptArgs a;
     std::memset(&a, 0, sizeof(a));
     a.batch = c->batch; a.K = c->K; a.w_tiles = c->D.w_tiles; a.m_cap = c->D.MC; a.vocab = c->D.vocab;
     a.stats = c->stats_t; a.stats_i = c->stats_it; a.logits = c->logits; a.dlogits = c->dlogits;
-    a.call = c->call; a.st = c->st;
+    a.call = call_of(c, seed, step, temperature > 0.f ? temperature : 1.0f, sample); a.st = c->st;
     a.page_table = c->m[0].page_table; a.pt_ld = c->D.pt_ld; a.page_size = c->lim.page_size;
     a.accept_len = d_accept_len; a.emitted = d_emitted; a.kv_slots = d_kv_slots; a.n_emit = d_n_emit;
     a.status = c->status;

@@ -407,6 +407,21 @@ __device__ __forceinline__ void store_pair4(__nv_bfloat16* x, int m, int col, in
   *reinterpret_cast<uint2*>(x + xpk(m, 1, col, x_rows)) = lv;
 }
 
+// Eight consecutive columns (col % 8 == 0): one 16-byte chunk in each of the
+// token's hi and lo rows.
+__device__ __forceinline__ void store_pair8(__nv_bfloat16* x, int m, int col, int x_rows, const float (&v)[8]) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    __nv_bfloat16 h0, l0, h1, l1;
+    split_bf16(v[2 * e], h0, l0);
+    split_bf16(v[2 * e + 1], h1, l1);
+    h[e] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
+    l[e] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+  }
+  *reinterpret_cast<uint4*>(x + xpk(m, 0, col, x_rows)) = make_uint4(h[0], h[1], h[2], h[3]);
+  *reinterpret_cast<uint4*>(x + xpk(m, 1, col, x_rows)) = make_uint4(l[0], l[1], l[2], l[3]);
+}
 __device__ __forceinline__ float silu(float z) { return z / (1.0f + expf(-z)); }
 
 // Warp reductions (fixed butterfly order, so results are deterministic).

@@ -285,6 +285,16 @@ __device__ __forceinline__ void epi_chunk(const GemmArgs& a, float (&v)[kEpiTok]
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (in[i]) *reinterpret_cast<float4*>(lp + epi_col(i, l8)) = x[i];
+      if (a.logits_out) {  // the caller's copy (a copy afterwards reads and writes the rows once more)
+        lp = a.logits_out + (size_t)orow * a.vocab + n0;
+        const bool vec = (reinterpret_cast<uintptr_t>(a.logits_out) & 15) == 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float* q = lp + epi_col(i, l8);
+          if (in[i] && vec) *reinterpret_cast<float4*>(q) = x[i];
+          else if (in[i]) { q[0] = x[i].x; q[1] = x[i].y; q[2] = x[i].z; q[3] = x[i].w; }
+        }
+      }
     }
     // tile max and argmax (lowest index on ties) of token jl
     float mv = -INFINITY;

@@ -76,6 +76,7 @@ struct GemmArgs {
   int hd, hkv, page_size, n_pages;
   // MODE_LOGITS
   float* logits;              // [rows_out][vocab] or null
+  float* logits_out;          // the caller's copy of them (null: none; any 4-byte alignment)
   const int* row_out;         // row -> output row, -1: none (null: identity)
   const int* row_gi;          // row -> Philox row index for Gumbel draws, -1: none
   float4* stats;              // [w_tiles][m_cap] {max, sumexp(T), gumbel best, 0}
@@ -162,6 +163,8 @@ struct EmbedArgs {
   float* ssq;
   int m_cap;
   uint32_t* status;
+  CallArgs call;               // the call's scalars, written to *call_out for the pass's other kernels (null: not)
+  CallArgs* call_out;
 };
 enum { EMB_PREFILL = 0, EMB_DRAFT = 1, EMB_VERIFY = 2, EMB_DRAFT_SEQ = 3 };
 
@@ -187,7 +190,7 @@ struct AcceptArgs {
   const int2* stats_i;
   const float* logits;     // [B][K+1][V] (sampling)
   const float* dlogits;    // [B][K][V] (sampling)
-  const CallArgs* call;
+  CallArgs call;
   DevState st;
   const int* page_table;
   int pt_ld, page_size;
@@ -211,9 +214,8 @@ struct GivenArgs {
   int sample;
   float4 *stats_t, *stats_d;
   int2* stats_it;
-  CallArgs call;           // written to *call_out with the reset state below
-  CallArgs* call_out;
-  DevState st;
+  CallArgs call;
+  DevState st;             // reset by block (0, 0)
   const int* d;            // [batch][K] candidates
   int batch, K;
 };

@@ -42,49 +42,80 @@ namespace pard {
 __global__ void __launch_bounds__(128) embed_kernel(const __grid_constant__ EmbedArgs a) {
   pdl_wait();
   pdl_trigger();
-  __shared__ int s_row0[65];
   __shared__ int s_tok;
   const int m = blockIdx.x;
-  if (threadIdx.x == 0) {
-    int total = 0;
+  if (threadIdx.x < 32) {
+    // Rows of each sequence and their prefix: two sequences a lane, all
+    // counts requested at once (one after the other they cost a memory
+    // latency per sequence).
+    const int lane = threadIdx.x;
+    int b = 0, row0 = 0, total = 0;
     if (a.mode == EMB_PREFILL) {
-      s_row0[0] = 0;
       total = a.pf_rows;
+      if (m == 0 && lane < 2) a.rp.seq_row0[lane] = lane ? total : 0;
     } else {
-      for (int b = 0; b < a.batch; ++b) {
-        s_row0[b] = total;
-        total += a.mode == EMB_DRAFT       ? a.st.pend_cnt[b] + a.K - 1
-                 : a.mode == EMB_DRAFT_SEQ ? (a.seq_i == 0 ? a.st.pend_cnt[b] : 1)
+      int cnt[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int sq = 2 * lane + e;
+        cnt[e] = sq >= a.batch ? 0
+                 : a.mode == EMB_DRAFT       ? a.st.pend_cnt[sq] + a.K - 1
+                 : a.mode == EMB_DRAFT_SEQ ? (a.seq_i == 0 ? a.st.pend_cnt[sq] : 1)
                                            : a.K + 1;
       }
-      s_row0[a.batch] = total;
+      int inc = cnt[0] + cnt[1];
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      total = __shfl_sync(0xffffffffu, inc, 31);
+      const int start = inc - cnt[0] - cnt[1];
+      if (m == 0) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          if (2 * lane + e < a.batch) a.rp.seq_row0[2 * lane + e] = start + (e ? cnt[0] : 0);
+        if (lane == 0) a.rp.seq_row0[a.batch] = total;
+      }
+      // this row's sequence: the last one that starts at or before it (an
+      // empty sequence starts where its successor does and is not the last)
+      int mine = -1, mine0 = 0;
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int at = start + (e ? cnt[0] : 0);
+        if (2 * lane + e < a.batch && at <= m) { mine = 2 * lane + e; mine0 = at; }
+      }
+      const unsigned has = __ballot_sync(0xffffffffu, mine >= 0);
+      const int src = 31 - __clz((int)has);
+      b = __shfl_sync(0xffffffffu, mine, src);
+      row0 = __shfl_sync(0xffffffffu, mine0, src);
     }
-    if (m == 0) {
+    if (m == 0 && lane == 0) {
       *a.rp.m_dev = total;
-      if (a.mode == EMB_PREFILL) { a.rp.seq_row0[0] = 0; a.rp.seq_row0[1] = total; }
-      else for (int b = 0; b <= a.batch; ++b) a.rp.seq_row0[b] = s_row0[b];
+      if (a.call_out) *a.call_out = a.call;
       if (total > a.m_cap) set_status(a.status, ST_BAD_ROWS);
     }
-    s_tok = -1;
+    int tok = -1;
     if (m < total && m < a.m_cap) {
-      int b = 0, j = m, tok = 0, pos = 0, out = -1, gi = -1;
+      int pos = 0, out = -1, gi = -1;
       if (a.mode == EMB_PREFILL) {
         b = a.pf_seq;
         tok = a.tokens[m];
         pos = a.pf_pos0 + m;
       } else {
-        while (b + 1 < a.batch && m >= s_row0[b + 1]) ++b;
-        j = m - s_row0[b];
-        const int n = a.st.n[b];
+        const int j = m - row0, kp = a.st.kmax + 1;
+        // the sequence's facts, requested together
+        const int n = a.st.n[b], p = a.st.pend_cnt[b];
+        const int pend = lane < kp ? a.st.pend[b * kp + lane] : 0;
         if (a.mode == EMB_DRAFT) {
-          const int p = a.st.pend_cnt[b];
-          tok = j < p ? a.st.pend[b * (a.st.kmax + 1) + j] : (a.mask_ids ? a.mask_ids[j - p] : a.mask_id);
+          const int mask = a.mask_ids ? a.mask_ids[max(0, min(j - p, a.K - 2))] : a.mask_id;
+          const int real = __shfl_sync(0xffffffffu, pend, min(j, 31));
+          tok = j < p ? real : mask;
           pos = n - p + j;
           if (j >= p - 1) { gi = j - (p - 1); out = b * a.K + gi; }
         } else if (a.mode == EMB_DRAFT_SEQ) {
-          const int p = a.st.pend_cnt[b];
           if (a.seq_i == 0) {
-            tok = a.st.pend[b * (a.st.kmax + 1) + j];
+            tok = __shfl_sync(0xffffffffu, pend, min(j, 31));
             pos = n - p + j;
             if (j == p - 1) { gi = 0; out = b * a.K; }
           } else {
@@ -94,41 +125,53 @@ __global__ void __launch_bounds__(128) embed_kernel(const __grid_constant__ Embe
             out = b * a.K + a.seq_i;
           }
         } else {
-          tok = j == 0 ? a.st.pend[b * (a.st.kmax + 1) + a.st.pend_cnt[b] - 1] : a.d_in[b * a.K + j - 1];
-          if (j > 0) a.st.d[b * a.st.kmax + j - 1] = tok;
+          const int cand = j > 0 ? a.d_in[b * a.K + j - 1] : 0;
+          const int last = __shfl_sync(0xffffffffu, pend, min(max(p - 1, 0), 31));
+          tok = j == 0 ? last : cand;
+          if (j > 0 && lane == 0) a.st.d[b * a.st.kmax + j - 1] = tok;
           pos = n - 1 + j;
           out = b * (a.K + 1) + j;
         }
       }
-      if (tok < 0 || tok >= a.vocab) { set_status(a.status, ST_BAD_TOKEN); tok = 0; }
-      a.rp.row_tok[m] = tok;
-      a.rp.row_pos[m] = pos;
-      a.rp.row_seq[m] = b;
-      a.rp.row_out[m] = out;
-      a.rp.row_gi[m] = gi;
-      s_tok = tok;
+      if (tok < 0 || tok >= a.vocab) {
+        if (lane == 0) set_status(a.status, ST_BAD_TOKEN);
+        tok = 0;
+      }
+      if (lane == 0) {
+        a.rp.row_tok[m] = tok;
+        a.rp.row_pos[m] = pos;
+        a.rp.row_seq[m] = b;
+        a.rp.row_out[m] = out;
+        a.rp.row_gi[m] = gi;
+      }
     }
+    if (lane == 0) s_tok = tok;
   }
   __syncthreads();
   const int tok = s_tok;
   if (tok < 0) return;
-  const __nv_bfloat16* e = a.embed + (size_t)tok * a.d;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int t = warp; t < a.d / 128; t += 4) {
-    float ss = 0.f;
+  const uint4* e = reinterpret_cast<const uint4*>(a.embed + (size_t)tok * a.d);
+  const uint4* g = reinterpret_cast<const uint4*>(a.gain0);
+  // a thread takes eight columns at a time, half a warp one 128-column tile
+  for (int c8 = threadIdx.x; c8 < a.d / 8; c8 += 128) {
+    const uint4 ev = e[c8], gv = g[c8];
+    const uint32_t ew[4] = {ev.x, ev.y, ev.z, ev.w}, gw[4] = {gv.x, gv.y, gv.z, gv.w};
+    float h[8], x[8], ss = 0.f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int c = t * 128 + lane * 4 + k;
-      const float h = __bfloat162float(e[c]);
-      a.h[(size_t)m * a.d + c] = h;
-      __nv_bfloat16 hi, lo;
-      split_bf16(h * __bfloat162float(a.gain0[c]), hi, lo);
-      a.x[xpk(m, 0, c, 2 * a.m_cap)] = hi;
-      a.x[xpk(m, 1, c, 2 * a.m_cap)] = lo;
-      ss += h * h;
+      h[2 * k] = __uint_as_float(ew[k] << 16);
+      h[2 * k + 1] = __uint_as_float(ew[k] & 0xffff0000u);
+      x[2 * k] = h[2 * k] * __uint_as_float(gw[k] << 16);
+      x[2 * k + 1] = h[2 * k + 1] * __uint_as_float(gw[k] & 0xffff0000u);
+      ss += h[2 * k] * h[2 * k] + h[2 * k + 1] * h[2 * k + 1];
     }
-    ss = warp_sum(ss);
-    if (lane == 0) a.ssq[(size_t)t * a.m_cap + m] = ss;
+    float4* hp = reinterpret_cast<float4*>(a.h + (size_t)m * a.d + c8 * 8);
+    hp[0] = make_float4(h[0], h[1], h[2], h[3]);
+    hp[1] = make_float4(h[4], h[5], h[6], h[7]);
+    store_pair8(a.x, m, c8 * 8, 2 * a.m_cap, x);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffu << (threadIdx.x & 16), ss, o, 16);
+    if ((threadIdx.x & 15) == 0) a.ssq[(size_t)(c8 >> 4) * a.m_cap + m] = ss;
   }
 }
 
@@ -424,7 +467,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) accept_test_kernel(const __gri
   __shared__ RowRed s_part[kRowWarps], s_row[17], s_drow[16];
   __shared__ float2 s_norm[17], s_dnorm[16];
   const int b = blockIdx.x;
-  const float T = a.call->temp;
+  const float T = a.call.temp;
   reduce_rows<true>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, T, s_part, s_row);
   if (a.dstats && a.K > 0)
     reduce_rows<true>(a.dstats, nullptr, a.w_tiles, a.d_m_cap, b * a.K, a.K, T, s_part, s_drow);
@@ -448,7 +491,7 @@ __global__ void __launch_bounds__(32 * kRowWarps) accept_test_kernel(const __gri
     const float2 zn = s_dnorm[i];
     const float zv = a.dlogits[((size_t)b * a.K + i) * a.vocab + di];
     const float q = expf(zv / T - zn.x / T) / zn.y;
-    const float u = uniform01(philox_word(a.call->seed, STREAM_ACCEPT, a.call->step, (uint32_t)b, (uint32_t)i, 0u));
+    const float u = uniform01(philox_word(a.call.seed, STREAM_ACCEPT, a.call.step, (uint32_t)b, (uint32_t)i, 0u));
     if (!(u * q < p)) { j = i; break; }
   }
   a.st.samp_a[b] = j;
@@ -467,7 +510,7 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
   __shared__ int s_i[256];
   __shared__ int s_last;
   const int b = blockIdx.x / kResampleSplit, part = blockIdx.x % kResampleSplit;
-  const float T = a.call->temp;
+  const float T = a.call.temp;
   const int j = a.st.samp_a[b];
   const float4 nm = a.st.samp_norm[b];
   const float* y = a.logits + ((size_t)b * (a.K + 1) + j) * a.vocab;
@@ -480,8 +523,8 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
   // before the logarithms: its score beats `best` only if -log u < w exp(-best)
   // (w exp(-best) = exp(y/T - best) without a draft row), and -log u >= 1 - u;
   // the factor 1.0001 is far above the roundings of both sides.
-  const uint64_t seed = a.call->seed;
-  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32), step = (uint32_t)a.call->step;
+  const uint64_t seed = a.call.seed;
+  const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32), step = (uint32_t)a.call.step;
   const float cy = nm.x / T, cz = nm.z / T;
   for (int blk0 = v0 / 4; 4 * blk0 < v1; blk0 += blockDim.x) {
     const int blk = blk0 + threadIdx.x;
@@ -554,7 +597,7 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
     float bb = -INFINITY;
     int bj = INT_MAX;
     for (int v = threadIdx.x; v < a.vocab; v += blockDim.x) {
-      const float g = gumbel(philox_word(a.call->seed, STREAM_BONUS, a.call->step, (uint32_t)b, 0u, (uint32_t)v));
+      const float g = gumbel(philox_word(a.call.seed, STREAM_BONUS, a.call.step, (uint32_t)b, 0u, (uint32_t)v));
       const float p = expf(y[v] / T - nm.x / T) / nm.y;
       argmax_merge(bb, bj, logf(p) + g, v);
     }
@@ -653,7 +696,7 @@ void launch_row_stats(const float* logits, int rows, int vocab, int w_tiles, int
 // Statistics of given logits rows in tiles of kGivenTile entries (max,
 // argmax, and when sampling the sum of exp((x - max)/T)): block (t, m) takes
 // tile t of row m, the target's rows first; block (0, 0) also resets the
-// acceptance state and writes the call's scalars.  HBM-bound: every logit is
+// acceptance state.  HBM-bound: every logit is
 // read once, 16 bytes a load, four loads in flight a thread (batch 16, K = 6:
 // 107 MB; the whole sampled acceptance 92 us, 231 us with one 512-byte tile a
 // block, three block reductions each and one row after the other after it; the
@@ -665,7 +708,6 @@ __global__ void __launch_bounds__(128) given_stats_kernel(const __grid_constant_
   const int m = target ? blockIdx.y : blockIdx.y - a.rows_t;
   const float* row = (target ? a.y : a.z) + (size_t)m * a.vocab;
   if (t == 0 && blockIdx.y == 0) {
-    if (tid == 0) *a.call_out = a.call;
     if (tid < a.batch) {
       a.st.n[tid] = 1;
       a.st.pend_cnt[tid] = 1;

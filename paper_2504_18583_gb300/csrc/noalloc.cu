@@ -28,8 +28,7 @@ constexpr int kNaRowsT = kNaMaxBatch * (kNaMaxK + 1);  // target rows: B (K+1)
 constexpr int kNaRowsD = kNaMaxBatch * kNaMaxK;        // draft rows: B K
 
 constexpr size_t al(size_t x) { return (x + 255) & ~size_t(255); }
-constexpr size_t kOffCall = 0;
-constexpr size_t kOffStatsT = al(kOffCall + sizeof(CallArgs));
+constexpr size_t kOffStatsT = 0;
 constexpr size_t kOffStatsIT = al(kOffStatsT + (size_t)kNaTiles * kNaRowsT * sizeof(float4));
 constexpr size_t kOffStatsD = al(kOffStatsIT + (size_t)kNaTiles * kNaRowsT * sizeof(int2));
 constexpr size_t kOffN = al(kOffStatsD + (size_t)kNaTiles * kNaRowsD * sizeof(float4));
@@ -110,7 +109,6 @@ extern "C" pard_status pard_accept_noalloc(const float* d_target_logits, const f
     return PARD_ERR_CUDA;
   }
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  CallArgs* call = reinterpret_cast<CallArgs*>(base + kOffCall);
   float4* stats_t = reinterpret_cast<float4*>(base + kOffStatsT);
   int2* stats_it = reinterpret_cast<int2*>(base + kOffStatsIT);
   float4* stats_d = reinterpret_cast<float4*>(base + kOffStatsD);
@@ -142,14 +140,13 @@ extern "C" pard_status pard_accept_noalloc(const float* d_target_logits, const f
     g.sample = sample ? 1 : 0;
     g.stats_t = stats_t; g.stats_d = stats_d; g.stats_it = stats_it;
     g.call = CallArgs{seed, step, temperature, sample ? 1 : 0, K, 0};
-    g.call_out = call;
     g.st = st; g.d = d_draft; g.batch = batch; g.K = K;
     launch_given_stats(g, s);
     AcceptArgs a;
     memset(&a, 0, sizeof(a));
     a.batch = batch; a.K = K; a.w_tiles = tiles; a.m_cap = kNaRowsT; a.vocab = vocab;
     a.stats = stats_t; a.stats_i = stats_it; a.logits = d_target_logits; a.dlogits = d_draft_logits;
-    a.call = call; a.st = st;
+    a.call = g.call; a.st = st;
     a.page_table = nullptr; a.pt_ld = 0; a.page_size = 16;
     a.accept_len = d_accept_len; a.emitted = d_emitted; a.kv_slots = nullptr; a.n_emit = nullptr;
     if (sample) {
