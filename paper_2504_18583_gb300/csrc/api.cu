@@ -336,13 +336,18 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
     const long w_pairs = (a.w_tiles + 1) / 2;
     const long units = w_pairs * a.tok_tiles * a.kc;
     if (2 * w_pairs * a.tok_tiles > kMaxGemmTiles || (units + 1) * (c->pairs + 1) > INT32_MAX) throw cudaErrorInvalidValue;
+    a.max_pairs = c->pairs;
     WideArgs w;
     w.g = a;
     const int buf = a.x == c->xd ? 0 : a.x == c->xo ? 1 : 2;
     w.x[0] = c->xmap[buf][a.n_tok / 16 - 1];
     w.x[1] = c->xmap[buf][kWideBoxL / 16 - 1];
     w.x[2] = c->xmap[buf][kWideBoxS / 16 - 1];
-    launch_gemm_wide(w, wide_pairs((int)units, a.kc, c->pairs), s, true);
+    // a pass with fewer rows than its capacity splits its fewer tiles anew
+    int pairs = 0;
+    for (int tiles = 1; tiles <= (a.m_early ? a.tok_tiles : 1); ++tiles)
+      pairs = std::max(pairs, wide_split((int)w_pairs * (a.m_early ? tiles : a.tok_tiles), a.kc, c->pairs).pairs);
+    launch_gemm_wide(w, pairs, s, true);
     c->launches++;
     return;
   }
@@ -364,9 +369,10 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
 // context).
 struct AttnGeom {
   int row_blocks, groups, n_split;
+  int prompt = 0;  // a prompt pass of many row blocks
   int nbuf;  // K/V chunk buffers of the attention kernel's form (4, or 2 for passes with many units)
 };
-AttnGeom attn_geometry(pard_ctx* c, int mi, int rows_per_seq, int batch) {
+AttnGeom attn_geometry(pard_ctx* c, int mi, int rows_per_seq, int batch, bool prompt) {
   const pard_model_cfg& cf = c->m[mi].cfg;
   const int rb_rows = attention_rows_per_block(cf.n_q_heads / cf.n_kv_heads);
   AttnGeom g;
@@ -375,6 +381,10 @@ AttnGeom attn_geometry(pard_ctx* c, int mi, int rows_per_seq, int batch) {
   const int n_kt = (c->lim.max_ctx + 31) / 32;  // 32-key chunks at the longest context
   g.n_split = std::max(1, std::min({c->attn_split_cap, n_kt, (2 * c->sm + g.groups - 1) / g.groups}));
   g.nbuf = 4;
+  if (prompt) {
+    g.prompt = 1;
+    return g;
+  }
   long total = 0, longest = 0;
   if (batch > 1 && (int)c->ctx_est.size() >= batch)
     for (int b = 0; b < batch; ++b) {
@@ -452,6 +462,7 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int batch
     a.page_size = c->lim.page_size; a.n_pages = c->lim.n_pages;
     a.row_blocks = geo.row_blocks; a.n_split = geo.n_split;
     a.nbuf = geo.nbuf;
+    a.prompt = geo.prompt;
     a.scale = (float)(1.4426950408889634 / std::sqrt((double)cf.head_dim));  // scores in units of log 2
     a.x_out = c->xo; a.x_rows = 2 * c->D.MC;
     a.status = c->status;
@@ -510,9 +521,9 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int batch
 // decomposition; pt_attn: page table row base the attention kernel indexes
 // by its sequence index.
 void run_layers(pard_ctx* c, int mi, int rows_cap, int batch, int rows_per_seq, const int* pt_attn,
-                cudaStream_t s, int fixed_rows = 0) {
+                cudaStream_t s, int fixed_rows = 0, bool prompt = false) {
   const int tt = pick_tt(rows_cap);
-  const AttnGeom geo = attn_geometry(c, mi, rows_per_seq, batch);
+  const AttnGeom geo = attn_geometry(c, mi, rows_per_seq, batch, prompt);
   for (int l = 0; l < c->m[mi].cfg.n_layers; ++l) {
     LayerPlan P = layer_plan(c, mi, l, rows_cap, tt, batch, pt_attn, geo, fixed_rows);
     // the pass's row count is written by the embedding kernel, which directly
@@ -867,7 +878,7 @@ pard_status pard_prefill(pard_ctx* c, const int32_t* d_tokens, const int32_t* h_
           e.pf_rows = rows;
           launch_embed(e, rows, s, true);
           c->launches++;
-          run_layers(c, mi, rows, 1, rows, M.page_table + (size_t)b * c->D.pt_ld, s);
+          run_layers(c, mi, rows, 1, rows, M.page_table + (size_t)b * c->D.pt_ld, s, 0, true);
           last_rows = rows;
         }
         if (mi == 0) {

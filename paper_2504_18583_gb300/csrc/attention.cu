@@ -45,9 +45,15 @@ __global__ void __launch_bounds__(kAttnThreads, NBUF == 2 ? (HD == 64 ? 5 : 4) :
   // before any partial is pushed)
   cluster_arrive_relaxed();
   const int group_idx = blockIdx.x / NS;
-  const int rb = group_idx % a.row_blocks;
-  const int kvh = (group_idx / a.row_blocks) % a.hkv;
-  const int b = group_idx / (a.row_blocks * a.hkv);
+  int rb = group_idx % a.row_blocks;
+  int kvh = (group_idx / a.row_blocks) % a.hkv;
+  int b = group_idx / (a.row_blocks * a.hkv);
+  if (a.prompt) {
+    // a prompt's later row blocks see more keys: the longest units first
+    kvh = group_idx % a.hkv;
+    b = (group_idx / a.hkv) % a.batch;
+    rb = a.row_blocks - 1 - group_idx / (a.hkv * a.batch);
+  }
   // Row plan, positions, page tables and the keys and values of earlier
   // passes are written before the previous kernel (the QKV projection), which
   // had itself waited for them before it let this grid start: the unit reads

@@ -12,7 +12,8 @@
 // halves the accumulator: two 256-column buffers, so one tile's epilogue runs
 // under the next tile's MMAs.
 //
-// The (tile, K-step) space is split evenly over the pairs.  A tile split
+// The tiles are shared out over the pairs whole, in equal parts or evenly by
+// K-steps, whichever is expected to end first (wide_split).  A tile split
 // between several pairs is finished by all of them: each stores its partial,
 // then finishes its own share of the tile's 16-token chunks, summing the
 // partials in pair order (deterministic).  (One finisher per tile gathers all
@@ -119,9 +120,10 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
   const int kc = a.kc;
   // unit indices: 32 bits (the host checks that U times the pairs fits; 64-bit
   // divisions made up half of a short launch's tail)
-  const int U = (a.w_tiles + 1) / 2 * tok_tiles * kc;
-  const int G = wide_pairs(U, kc, (int)(gridDim.x >> 1));  // pairs with work
-  auto start_of = [&](int cc) { return cc * U / G; };
+  const int T = (a.w_tiles + 1) / 2 * tok_tiles, U = T * kc;
+  const WideSplit split = wide_split(T, kc, a.max_pairs);
+  const int G = split.pairs;  // pairs with work
+  auto start_of = [&](int cc) { return split.tiles ? cc * T / G * kc : cc * U / G; };
   auto owner = [&](int u) { return ((u + 1) * G + U - 1) / U - 1; };
   const int u0 = c < G ? start_of(c) : 0, u1 = c < G ? start_of(c + 1) : 0;
   const uint32_t b_bytes = (uint32_t)n_tok * 128;  // half of the tile's tokens, hi and lo rows
@@ -363,15 +365,18 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         if (!whole) {
           const int slot = ub == u0 ? 0 : 1;
           float* mine = a.partials + ((size_t)(2 * c + rank) * 2 + slot) * kTileF;
-#pragma unroll 2
-          for (int ch = grp; ch < nch; ch += 2) {
-            float v[kEpiTok];
-            load_acc(tbase + ch * kEpiTok, v);
+          // two chunks a turn: one accumulator read for both
+#pragma unroll 1
+          for (int ch = 2 * grp; ch < nch; ch += 4) {
+            uint32_t r[32];
+            tmem_ld32(tbase + ch * kEpiTok, r);
             // [chunk][j4][row] float4s: a warp's stores are 512 contiguous bytes
             float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kChF) + fr;
 #pragma unroll
-            for (int j4 = 0; j4 < 4; ++j4)
-              dst[j4 * kTileN] = make_float4(v[4 * j4], v[4 * j4 + 1], v[4 * j4 + 2], v[4 * j4 + 3]);
+            for (int j4 = 0; j4 < 8; ++j4)
+              if (j4 < 4 || ch + 1 < nch)
+                dst[j4 * kTileN] = make_float4(__uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
+                                               __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
           }
           tc_fence_before();
           all_epi_bar();  // orders every thread's partial before the one release OR

@@ -51,6 +51,7 @@ struct GemmArgs {
   float* partials;
   int* counters;              // split-K arrival masks: 64-bit word per output tile, zero between launches
   uint32_t* status;
+  int max_pairs;              // wide GEMM: pairs the GPU holds at once
   int stages;                 // ring slots used (0: all the kernel has)
   int pre_stages;             // slots filled before waiting on the previous kernel (0: stages)
   // RMS row scale applied after the reduction (null: none)
@@ -101,6 +102,7 @@ struct AttnArgs {
   int hq, hkv, hd, page_size, n_pages;
   int row_blocks;             // row blocks per sequence (grid.y / ...)
   int n_split;                // key splits
+  int prompt;                 // a prompt pass: units are launched longest first
   int nbuf;                   // K/V chunk buffers a CTA keeps (4, or 2 for ragged or crowded passes)
   float scale;                // log2(e) / sqrt(hd)
   __nv_bfloat16* x_out;       // packed [2*rows][hq*hd] hi/lo
@@ -239,12 +241,35 @@ __host__ __device__ inline void wide_tiles(int m, int& tiles, int& n_tok) {
   tiles = (m + kWideTok - 1) / kWideTok;
   n_tok = ((m + tiles - 1) / tiles + 15) / 16 * 16;
 }
-// Pairs that share U units: at least four units (64 KB of weights a CTA) each,
-// and no more than 56 to a tile of kc units.
-__host__ __device__ inline int wide_pairs(int U, int kc, int max_pairs) {
+// How T tiles of kc units (64 columns of K) are shared out over at most
+// max_pairs pairs: evenly by units (a pair may begin and end inside a tile),
+// or with tiles whole, or each cut into the same number of parts.  Finishing
+// a split tile costs a launch about kWideExchange units of time on top of its
+// epilogue, and a pair with two split tiles kWideSecond more than with one, so
+// the even split has to save more than that.  Measured (batch-16 draft and
+// verify of 8 layers, 512-row prompt; us): always even 1673 / 1497 / 18007,
+// with equal parts 1643 / 1426 / 17422, with whole tiles too 1549 / 1384 / 16785
+// at (40, 8); 1566 / 1444 / 16999 at (12, 4), 1562 / 1387 / 16899 at (64, 8).
+// Fewer tiles than pairs stay whole only up to kWideWhole units: the tensor
+// cores truncate at every accumulation (hi and lo parts: eight a unit), and
+// with the QKV projection's 64 units in one accumulator the keys' and values'
+// bf16 roundings moved the error of 6 layers over a 512-row prompt from
+// 1.36e-3 to 1.57e-3 (1.38e-3 with the even split, at the same speed).
+constexpr int kWideExchange = 40, kWideSecond = 8, kWideWhole = 32;
+struct WideSplit {
+  int pairs;
+  bool tiles;  // ranges are whole tiles
+};
+__host__ __device__ inline WideSplit wide_split(int T, int kc, int max_pairs) {
+  // at least four units (64 KB of weights a CTA) a pair, and at most 56 pairs to a tile
   const int least = kc > 4 * 54 ? (kc + 53) / 54 : 4;
-  const int n = U / least;
-  return n < 1 ? 1 : (n < max_pairs ? n : max_pairs);
+  const int most = T * kc / least < 1 ? 1 : (T * kc / least < max_pairs ? T * kc / least : max_pairs);
+  const int even = (T * kc + most - 1) / most;
+  if (T >= most) return {most, (T + most - 1) / most * kc <= even + kWideExchange};
+  const int parts = most / T;
+  if (parts == 1 && kc <= kWideWhole) return {T, true};
+  if (parts > 1 && (kc + parts - 1) / parts <= even + kWideSecond) return {T * parts, false};
+  return {most, false};
 }
 
 // launchers (gemm.cu, gemm_wide.cu, attention.cu, misc.cu)
