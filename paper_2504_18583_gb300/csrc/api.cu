@@ -372,7 +372,8 @@ struct AttnGeom {
   int prompt = 0;  // a prompt pass of many row blocks
   int nbuf;  // K/V chunk buffers of the attention kernel's form (4, or 2 for passes with many units)
 };
-AttnGeom attn_geometry(pard_ctx* c, int mi, int rows_per_seq, int batch, bool prompt) {
+// units: of a prompt pass (0: a decode pass), the (sequence, row block) pairs that hold rows.
+AttnGeom attn_geometry(pard_ctx* c, int mi, int rows_per_seq, int batch, int units) {
   const pard_model_cfg& cf = c->m[mi].cfg;
   const int rb_rows = attention_rows_per_block(cf.n_q_heads / cf.n_kv_heads);
   AttnGeom g;
@@ -381,8 +382,10 @@ AttnGeom attn_geometry(pard_ctx* c, int mi, int rows_per_seq, int batch, bool pr
   const int n_kt = (c->lim.max_ctx + 31) / 32;  // 32-key chunks at the longest context
   g.n_split = std::max(1, std::min({c->attn_split_cap, n_kt, (2 * c->sm + g.groups - 1) / g.groups}));
   g.nbuf = 4;
-  if (prompt) {
+  if (units > 0) {
     g.prompt = 1;
+    const int live = units * cf.n_kv_heads;
+    g.n_split = std::max(1, std::min({c->attn_split_cap, n_kt, (2 * c->sm + live - 1) / live}));
     return g;
   }
   long total = 0, longest = 0;
@@ -521,9 +524,9 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int batch
 // decomposition; pt_attn: page table row base the attention kernel indexes
 // by its sequence index.
 void run_layers(pard_ctx* c, int mi, int rows_cap, int batch, int rows_per_seq, const int* pt_attn,
-                cudaStream_t s, int fixed_rows = 0, bool prompt = false) {
+                cudaStream_t s, int fixed_rows = 0, int prompt_units = 0) {
   const int tt = pick_tt(rows_cap);
-  const AttnGeom geo = attn_geometry(c, mi, rows_per_seq, batch, prompt);
+  const AttnGeom geo = attn_geometry(c, mi, rows_per_seq, batch, prompt_units);
   for (int l = 0; l < c->m[mi].cfg.n_layers; ++l) {
     LayerPlan P = layer_plan(c, mi, l, rows_cap, tt, batch, pt_attn, geo, fixed_rows);
     // the pass's row count is written by the embedding kernel, which directly
@@ -862,32 +865,46 @@ pard_status pard_prefill(pard_ctx* c, const int32_t* d_tokens, const int32_t* h_
     for (int b = 0; b < batch; ++b) c->ctx_est[b] = h_lens[b] + n_new;
     c->prefilled = false;
     set_call(c, seed, 0, temperature, sample, s);
+    // The prompts are one run of rows, a sequence after the other: every pass
+    // takes the next prefill_chunk of them, whichever sequences they belong to
+    // (a pass per sequence streams all weights for each short prompt).
     const int chunk = c->lim.prefill_chunk;
-    long offset = 0;
-    for (int b = 0; b < batch; ++b) {
-      const int len = h_lens[b];
-      for (int mi = 0; mi < 2; ++mi) {
-        Model& M = c->m[mi];
-        int last_rows = 0;
-        for (int start = 0; start < len; start += chunk) {
-          const int rows = std::min(chunk, len - start);
-          EmbedArgs e = embed_base(c, mi, EMB_PREFILL);
-          e.tokens = d_tokens + offset + start;
-          e.pf_seq = b;
-          e.pf_pos0 = start;
-          e.pf_rows = rows;
-          launch_embed(e, rows, s, true);
-          c->launches++;
-          run_layers(c, mi, rows, 1, rows, M.page_table + (size_t)b * c->D.pt_ld, s, 0, true);
-          last_rows = rows;
+    std::vector<long> off(batch + 1, 0);
+    for (int b = 0; b < batch; ++b) off[b + 1] = off[b] + h_lens[b];
+    const long total = off[batch];
+    for (int mi = 0; mi < 2; ++mi) {
+      Model& M = c->m[mi];
+      const int rb_rows = attention_rows_per_block(M.cfg.n_q_heads / M.cfg.n_kv_heads);
+      int b0 = 0;
+      for (long r0 = 0; r0 < total; r0 += chunk) {
+        const int rows = (int)std::min<long>(chunk, total - r0);
+        while (off[b0 + 1] <= r0) ++b0;
+        int b1 = b0, most = 0, units = 0;
+        GatherArgs g;
+        for (; b1 < batch && off[b1] < r0 + rows; ++b1) {
+          const int n = (int)(std::min(off[b1 + 1], r0 + rows) - std::max(off[b1], r0));
+          most = std::max(most, n);
+          units += (n + rb_rows - 1) / rb_rows;
+          g.src[b1 - b0] = off[b1 + 1] <= r0 + rows ? (int)(off[b1 + 1] - 1 - r0) : -1;  // the prompt's last row
         }
+        EmbedArgs e = embed_base(c, mi, EMB_PREFILL);
+        e.tokens = d_tokens;
+        e.plen = c->g_plen;
+        e.pf_row0 = (int)r0;
+        e.pf_rows = rows;
+        e.pf_seq = b0;
+        e.pf_nseq = b1 - b0;
+        launch_embed(e, rows, s, true);
+        c->launches++;
+        run_layers(c, mi, rows, b1 - b0, most, M.page_table + (size_t)b0 * c->D.pt_ld, s, 0, units);
         if (mi == 0) {
-          launch_gather_rows(c->xd, 2 * c->D.MC, c->ssq, M.cfg.d_model / 128, c->D.MC, last_rows - 1, c->xg,
-                             2 * c->D.gcap, c->ssqg, c->D.MC, b, M.cfg.d_model, s, true);
+          g.x = c->xd; g.ssq = c->ssq; g.xg = c->xg; g.ssqg = c->ssqg;
+          g.x_rows = 2 * c->D.MC; g.xg_rows = 2 * c->D.gcap; g.ssq_tiles = M.cfg.d_model / 128;
+          g.m_cap_src = c->D.MC; g.m_cap_dst = c->D.MC; g.d = M.cfg.d_model; g.dst0 = b0;
+          launch_gather_rows(g, b1 - b0, s, true);
           c->launches++;
         }
       }
-      offset += len;
     }
     const int gtt = pick_tt(c->D.gcap);
     run_lm_head(c, 0, c->xg, 2 * c->D.gcap, c->ssqg, batch, gtt, c->g_m, nullptr, nullptr, nullptr, sample ? c->g_row_gi : nullptr,

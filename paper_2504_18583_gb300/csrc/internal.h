@@ -155,8 +155,10 @@ struct EmbedArgs {
   const int* mask_ids;  // EMB_DRAFT: id of mask m_k per offset k (null: mask_id for all)
   const __nv_bfloat16* embed;
   const __nv_bfloat16* gain0;  // first layer's attention-norm gain
-  const int* tokens;           // prefill: this chunk's tokens
-  int pf_seq, pf_pos0, pf_rows;
+  const int* tokens;           // prefill: the prompts, concatenated
+  const int* plen;             // prefill: their lengths
+  int pf_row0, pf_rows;        // prefill: this pass's first row of the concatenation, its rows,
+  int pf_seq, pf_nseq;         // its first sequence and the number of sequences it touches
   const int* d_in;             // verify: candidates to feed ([B][K])
   DevState st;
   RowPlan rp;
@@ -274,9 +276,16 @@ __host__ __device__ inline WideSplit wide_split(int T, int kc, int max_pairs) {
 
 // launchers (gemm.cu, gemm_wide.cu, attention.cu, misc.cu)
 void launch_embed(const EmbedArgs& a, int grid, cudaStream_t s, bool pdl);
-void launch_gather_rows(const __nv_bfloat16* x, int x_rows, const float* ssq, int ssq_tiles, int m_cap_src, int src_row,
-                        __nv_bfloat16* xg, int xg_rows, float* ssqg, int m_cap_dst, int dst_row, int d, cudaStream_t s,
-                        bool pdl);
+constexpr int kMaxBatch = 64;
+struct GatherArgs {            // row src[i] of x and of its sums of squares to row dst0 + i (src[i] < 0: none)
+  const __nv_bfloat16* x;
+  const float* ssq;
+  __nv_bfloat16* xg;
+  float* ssqg;
+  int x_rows, xg_rows, ssq_tiles, m_cap_src, m_cap_dst, d, dst0;
+  int src[kMaxBatch];
+};
+void launch_gather_rows(const GatherArgs& a, int n, cudaStream_t s, bool pdl);
 void launch_pack(const __nv_bfloat16* tmp, __nv_bfloat16* w, int R, int K, int nblocks, bool unpack, cudaStream_t s);
 void launch_select(const SelectArgs& a, cudaStream_t s, bool pdl);
 void launch_given_stats(const GivenArgs& a, cudaStream_t s);

@@ -35,7 +35,7 @@ namespace pard {
 //   sequential draft (vanilla speculative decoding), pass i: i = 0 feeds
 //                   the pending real tokens (logits row: the last), i > 0
 //                   feeds candidate d_{i-1} at position n-1+i;
-//   prefill:        a chunk of one sequence's prompt.
+//   prefill:        a run of rows of the concatenated prompts.
 // h = E[token]; x = h * g (hi/lo bf16 pairs); ssq[t][m] = sum of h^2 over
 // the 128 columns of tile t.
 // ---------------------------------------------------------------------------
@@ -50,16 +50,15 @@ __global__ void __launch_bounds__(128) embed_kernel(const __grid_constant__ Embe
     // latency per sequence).
     const int lane = threadIdx.x;
     int b = 0, row0 = 0, total = 0;
-    if (a.mode == EMB_PREFILL) {
-      total = a.pf_rows;
-      if (m == 0 && lane < 2) a.rp.seq_row0[lane] = lane ? total : 0;
-    } else {
+    {
+      const bool prompt = a.mode == EMB_PREFILL;
       int cnt[2];
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
         const int sq = 2 * lane + e;
         cnt[e] = sq >= a.batch ? 0
-                 : a.mode == EMB_DRAFT       ? a.st.pend_cnt[sq] + a.K - 1
+                 : prompt                  ? a.plen[sq]
+                 : a.mode == EMB_DRAFT     ? a.st.pend_cnt[sq] + a.K - 1
                  : a.mode == EMB_DRAFT_SEQ ? (a.seq_i == 0 ? a.st.pend_cnt[sq] : 1)
                                            : a.K + 1;
       }
@@ -69,13 +68,18 @@ __global__ void __launch_bounds__(128) embed_kernel(const __grid_constant__ Embe
         const int v = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= o) inc += v;
       }
-      total = __shfl_sync(0xffffffffu, inc, 31);
-      const int start = inc - cnt[0] - cnt[1];
+      total = prompt ? a.pf_rows : __shfl_sync(0xffffffffu, inc, 31);
+      // first row of the lane's sequences in this pass (a prompt pass is a run
+      // of rows of all prompts, one after the other; negative: it began earlier)
+      const int start = inc - cnt[0] - cnt[1] - (prompt ? a.pf_row0 : 0);
       if (m == 0) {
+        const int s0 = prompt ? a.pf_seq : 0, ns = prompt ? a.pf_nseq : a.batch;
 #pragma unroll
-        for (int e = 0; e < 2; ++e)
-          if (2 * lane + e < a.batch) a.rp.seq_row0[2 * lane + e] = start + (e ? cnt[0] : 0);
-        if (lane == 0) a.rp.seq_row0[a.batch] = total;
+        for (int e = 0; e < 2; ++e) {
+          const int i = 2 * lane + e - s0;
+          if (i >= 0 && i < ns) a.rp.seq_row0[i] = max(0, start + (e ? cnt[0] : 0));
+        }
+        if (lane == 0) a.rp.seq_row0[ns] = total;
       }
       // this row's sequence: the last one that starts at or before it (an
       // empty sequence starts where its successor does and is not the last)
@@ -99,9 +103,8 @@ __global__ void __launch_bounds__(128) embed_kernel(const __grid_constant__ Embe
     if (m < total && m < a.m_cap) {
       int pos = 0, out = -1, gi = -1;
       if (a.mode == EMB_PREFILL) {
-        b = a.pf_seq;
-        tok = a.tokens[m];
-        pos = a.pf_pos0 + m;
+        tok = a.tokens[a.pf_row0 + m];
+        pos = m - row0;
       } else {
         const int j = m - row0, kp = a.st.kmax + 1;
         // the sequence's facts, requested together
@@ -197,25 +200,23 @@ void launch_embed(const EmbedArgs& a, int grid, cudaStream_t s, bool pdl) {
   PARD_LAUNCH(embed_kernel, grid, 128, 0, s, pdl, a);
 }
 
-// Copy one activation row (hi/lo pair, packed layout) and its sum-of-squares partials.
-__global__ void gather_rows_kernel(const __nv_bfloat16* x, int x_rows, const float* ssq, int ssq_tiles, int m_cap_src,
-                                   int src_row, __nv_bfloat16* xg, int xg_rows, float* ssqg, int m_cap_dst, int dst_row,
-                                   int d) {
+// Copy activation rows (hi/lo pairs, packed layout) and their sum-of-squares partials.
+__global__ void __launch_bounds__(256) gather_rows_kernel(const __grid_constant__ GatherArgs a) {
   pdl_wait();
   pdl_trigger();
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    xg[xpk(dst_row, 0, c, xg_rows)] = x[xpk(src_row, 0, c, x_rows)];
-    xg[xpk(dst_row, 1, c, xg_rows)] = x[xpk(src_row, 1, c, x_rows)];
+  const int src = a.src[blockIdx.x], dst = a.dst0 + blockIdx.x;
+  if (src < 0) return;
+  for (int i = threadIdx.x; i < a.d / 4; i += blockDim.x) {  // 8 columns of the hi or the lo row
+    const int c = i / 2 * 8, lo = i & 1;
+    *reinterpret_cast<uint4*>(a.xg + xpk(dst, lo, c, a.xg_rows)) =
+        *reinterpret_cast<const uint4*>(a.x + xpk(src, lo, c, a.x_rows));
   }
-  for (int t = threadIdx.x; t < ssq_tiles; t += blockDim.x)
-    ssqg[(size_t)t * m_cap_dst + dst_row] = ssq[(size_t)t * m_cap_src + src_row];
+  for (int t = threadIdx.x; t < a.ssq_tiles; t += blockDim.x)
+    a.ssqg[(size_t)t * a.m_cap_dst + dst] = a.ssq[(size_t)t * a.m_cap_src + src];
 }
 
-void launch_gather_rows(const __nv_bfloat16* x, int x_rows, const float* ssq, int ssq_tiles, int m_cap_src, int src_row,
-                        __nv_bfloat16* xg, int xg_rows, float* ssqg, int m_cap_dst, int dst_row, int d, cudaStream_t s,
-                        bool pdl) {
-  PARD_LAUNCH(gather_rows_kernel, 1, 256, 0, s, pdl, x, x_rows, ssq, ssq_tiles, m_cap_src, src_row, xg, xg_rows, ssqg,
-              m_cap_dst, dst_row, d);
+void launch_gather_rows(const GatherArgs& a, int n, cudaStream_t s, bool pdl) {
+  PARD_LAUNCH(gather_rows_kernel, n, 256, 0, s, pdl, a);
 }
 
 // Weight packing: nblocks consecutive R-row blocks of a [N][K] matrix move

@@ -508,3 +508,17 @@ def test_wide_gemm_tile_edges(batch, K, lens, chunk):
         greedy_step(P, step)
     assert P.eng.last_status() == 0
     print("stats", P.stats)
+
+
+@pytest.mark.parametrize("lens", [(1, 64, 63, 2, 130), (200, 1, 1, 1), (64, 64, 1)])
+def test_prompts_of_several_sequences_in_one_pass(lens):
+    """Prompt passes take 64 rows of the concatenated prompts at a time:
+    prompts that begin, end and continue inside a pass, one-token prompts and
+    prompts of exactly a pass; first tokens, then two greedy steps."""
+    wl = S.WORKLOADS["tiny"].replace(batch=len(lens), prompt_len=None, prompt_lens_given=lens, n_new=12)
+    P = Pair(wl, prefill_chunk=64)
+    P.prefill()
+    for step in range(1, 3):
+        greedy_step(P, step)
+    assert P.eng.last_status() == 0
+    print("stats", P.stats)
