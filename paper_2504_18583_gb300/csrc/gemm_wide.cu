@@ -126,6 +126,14 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
   auto start_of = [&](int cc) { return split.tiles ? cc * T / G * kc : cc * U / G; };
   auto owner = [&](int u) { return ((u + 1) * G + U - 1) / U - 1; };
   const int u0 = c < G ? start_of(c) : 0, u1 = c < G ? start_of(c + 1) : 0;
+  // QKV: this pair's share [tb, te) of the tile of unit u is summed in pieces
+  // of equal length, at most `chain` units each: the end of u's piece.
+  auto piece_end = [&](int u, int tb, int te) {
+    if constexpr (MODE != MODE_QKV) return te;
+    const int chain = n_tok > 128 ? kWideChainPrompt : kWideChain;
+    const int pieces = (te - tb + chain - 1) / chain, len = (te - tb + pieces - 1) / pieces;
+    return min(tb + ((u - tb) / len + 1) * len, te);
+  };
   const uint32_t b_bytes = (uint32_t)n_tok * 128;  // half of the tile's tokens, hi and lo rows
   const uint32_t stage_bytes = (uint32_t)kTileN * 128 + b_bytes;
   const int R = min(kWideMaxStages, kWideRing / (int)stage_bytes);
@@ -245,7 +253,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
       int seg_i = 0;
       bool ok = true;
       for (int u = u0; u < u1 && ok;) {
-        const int ub = u, ue = min((u / kc + 1) * kc, u1);
+        const int tile0 = u / kc * kc;
+        const int ub = u, ue = piece_end(u, max(tile0, u0), min(tile0 + kc, u1));
         const int ab = seg_i & 1;
         ok = __all_sync(0xffffffffu, mbar_wait_cluster(&acce[ab], (uint32_t)((seg_i >> 1) & 1) ^ 1u, abort_flag));
         if (!ok) break;
@@ -340,19 +349,27 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
       int take0 = 0, take1 = 0, base1 = 0;  // chunks of this turn: of the tile / first share, of the second share
       bool staged = true;
       unsigned long long old0 = 0, old1 = 0;
+      const float* sum = nullptr;  // from the accumulator: what earlier pieces of the tile added up to
       uint32_t tbase = 0;
       int wt0 = 0, wt1 = 0, tb0 = 0, tb1 = 0, n0 = 0, n1 = 0, ch0 = 0, ch1 = 0;  // tile, token, contributors, first chunk
       int ab = 0;
       if (from_acc) {
         const int t = u / kc;
-        const int ub = u, ue = min((t + 1) * kc, u1);
+        const int tb = max(t * kc, u0), te = min((t + 1) * kc, u1);
+        const int ub = u, ue = piece_end(u, tb, te);
         u = ue;
         ab = seg_i & 1;
         wt0 = 2 * (t / tok_tiles) + (int)rank;
         tb0 = t % tok_tiles * n_tok;
         const int nch = chunks_of(wt0, tb0);
-        const bool whole = ub == t * kc && ue == (t + 1) * kc;
-        if (whole) take0 = nch;
+        const bool whole = tb == t * kc && te == (t + 1) * kc;
+        const bool last = ue == te;
+        if (whole && last) take0 = nch;
+        // this pair's sum so far, or its partial; a whole tile's is gone
+        // before the range's last tile, which may be split, begins
+        const int slot = !whole && tb == u0 ? 0 : 1;
+        float* mine = a.partials + ((size_t)(2 * c + rank) * 2 + slot) * kTileF;
+        sum = ub > tb ? mine : nullptr;
         ok = mbar_wait(&accf[ab], (uint32_t)((seg_i >> 1) & 1), abort_flag);
         if (all_epi_any(!ok)) {
           if (et256 == 0) set_status(a.status, ST_TIMEOUT_EPI);
@@ -362,9 +379,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         ++seg_i;
         tc_fence_after();
         tbase = tmem + ab * kWideTok + ((uint32_t)(q * 32) << 16);
-        if (!whole) {
-          const int slot = ub == u0 ? 0 : 1;
-          float* mine = a.partials + ((size_t)(2 * c + rank) * 2 + slot) * kTileF;
+        if (!whole || !last) {
           // two chunks a turn: one accumulator read for both
 #pragma unroll 1
           for (int ch = 2 * grp; ch < nch; ch += 4) {
@@ -374,13 +389,22 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
             float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kChF) + fr;
 #pragma unroll
             for (int j4 = 0; j4 < 8; ++j4)
-              if (j4 < 4 || ch + 1 < nch)
-                dst[j4 * kTileN] = make_float4(__uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
-                                               __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
+              if (j4 < 4 || ch + 1 < nch) {
+                float4 f = make_float4(__uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
+                                       __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
+                if (MODE == MODE_QKV && sum) {
+                  const float4 o = __ldcg(dst + j4 * kTileN);  // this thread's own
+                  f = make_float4(f.x + o.x, f.y + o.y, f.z + o.z, f.w + o.w);
+                }
+                dst[j4 * kTileN] = f;
+              }
           }
           tc_fence_before();
-          all_epi_bar();  // orders every thread's partial before the one release OR
+          // orders every thread's partial before the one release OR, and
+          // before another thread's reads of a whole tile's sum
+          all_epi_bar();
           if (et == 0) mbar_arrive_remote(&acce[ab], 0);
+          if (!last) continue;
           const int cf = owner(t * kc), n = owner((t + 1) * kc - 1) - cf + 1, i = c - cf;
           if (et256 == 0 && nch > 0) red_release_or64(mask_of(t), 1ull << i);
           const Share h{t, wt0, tb0, cf, n, min(n, nch), (i * nch + n - 1) / n, ((i + 1) * nch + n - 1) / n};
@@ -481,6 +505,17 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         float v[kEpiTok];
         if (from_acc) {
           load_acc(tbase + i * kEpiTok, v);
+          if (MODE == MODE_QKV && sum) {
+            const float4* p = reinterpret_cast<const float4*>(sum + (size_t)i * kChF) + fr;
+#pragma unroll
+            for (int j4 = 0; j4 < 4; ++j4) {
+              const float4 pv = __ldcg(p + j4 * kTileN);
+              v[4 * j4 + 0] += pv.x;
+              v[4 * j4 + 1] += pv.y;
+              v[4 * j4 + 2] += pv.z;
+              v[4 * j4 + 3] += pv.w;
+            }
+          }
         } else {
 #pragma unroll
           for (int j = 0; j < kEpiTok; ++j) v[j] = 0.f;

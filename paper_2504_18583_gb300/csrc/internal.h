@@ -232,6 +232,15 @@ constexpr int kMaxAttnSplit = 16;       // key splits (CTAs of one cluster) of o
 // rows and at most kWideTok tokens, multiplied by a pair of CTAs.
 constexpr int kWideTok = 256;
 constexpr int kWideReadShift = 56;  // a split tile's mask word: 56 contributors, and above them its finished shares
+// Units of the QKV projection that one accumulator sums before the epilogue
+// adds it up in fp32 registers: the tensor cores truncate at every
+// accumulation (hi and lo parts: eight a unit), and keys and values are
+// rounded to bf16 afterwards, so that small differences become whole
+// roundings.  Error against 64 bits, 4 layers of the 8B widths over a 512-row
+// prompt: 1.08e-3 with one accumulator per part and 64-token tiles, 1.11e-3
+// without a limit here, 1.02e-3 at 24 units, 0.99e-3 at 16 (the whole pass
+// 0.7% slower); a decode pass's 21 units stay in one piece.
+constexpr int kWideChain = 24, kWideChainPrompt = 16;
 constexpr int kWideMaxRows = 2048;  // rows of one pass (64 sequences x 2 x 16)
 constexpr int kWideBoxL = 32, kWideBoxS = 16;
 struct WideArgs {
