@@ -213,7 +213,7 @@ constexpr int kGivenTile = 2048;
 struct GivenArgs {
   const float* y;          // [rows_t][vocab]
   const float* z;          // [rows_d][vocab] (rows_d = 0: none)
-  int rows_t, rows_d, m_cap_t, m_cap_d, vocab;
+  int rows_t, rows_d, m_cap_t, m_cap_d, vocab, tiles;
   int vec;                 // both arrays are 16-byte aligned
   int sample;
   float4 *stats_t, *stats_d;

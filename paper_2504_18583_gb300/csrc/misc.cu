@@ -276,41 +276,62 @@ __device__ __forceinline__ void merge_red(RowRed& r, const RowRed& o, float T) {
   argmax_merge(r.gv, r.gi, o.gv, o.gi);
 }
 
-// Block-wide reduction over the w_tiles tile statistics of one row; every
-// thread returns the result.  Fixed order: strided per thread, then a tree.
+// Block-wide reduction (256 threads) over the w_tiles tile statistics of one
+// row; thread 0 returns the result.  Fixed order: strided per thread with all
+// loads in flight, a shuffle tree per warp, then the warps in order.
 __device__ RowRed reduce_row(const float4* stats, const int2* stats_i, int w_tiles, int m_cap, int m, float T,
                              RowRed* sred) {
   RowRed r{-INFINITY, INT_MAX, 0.f, -INFINITY, INT_MAX};
-  for (int t = threadIdx.x; t < w_tiles; t += blockDim.x) {
-    const float4 s = stats[(size_t)t * m_cap + m];
-    const int2 si = stats_i[(size_t)t * m_cap + m];
-    RowRed o{s.x, si.x, s.y, s.z, si.y < 0 ? INT_MAX : si.y};
-    merge_red(r, o, T);
+  for (int t0 = threadIdx.x; t0 < w_tiles; t0 += 4 * 256) {
+    float4 s[4];
+    int2 si[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const size_t at = (size_t)min(t0 + k * 256, w_tiles - 1) * m_cap + m;
+      s[k] = stats[at];
+      si[k] = stats_i[at];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (t0 + k * 256 < w_tiles) merge_red(r, RowRed{s[k].x, si[k].x, s[k].y, s[k].z, si[k].y < 0 ? INT_MAX : si[k].y}, T);
   }
-  sred[threadIdx.x] = r;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) merge_red(sred[threadIdx.x], sred[threadIdx.x + w], T);
-    __syncthreads();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    RowRed x;
+    x.mx = __shfl_xor_sync(0xffffffffu, r.mx, o);
+    x.arg = __shfl_xor_sync(0xffffffffu, r.arg, o);
+    x.se = __shfl_xor_sync(0xffffffffu, r.se, o);
+    x.gv = __shfl_xor_sync(0xffffffffu, r.gv, o);
+    x.gi = __shfl_xor_sync(0xffffffffu, r.gi, o);
+    merge_red(r, x, T);
   }
-  RowRed out = sred[0];
+  if ((threadIdx.x & 31) == 0) sred[threadIdx.x >> 5] = r;
   __syncthreads();
-  return out;
+  r = sred[0];
+  if (threadIdx.x == 0)
+    for (int w = 1; w < 8; ++w) merge_red(r, sred[w], T);
+  return r;
 }
 
-// The same for rows m0 .. m0 + nrows - 1 at once (nrows <= 32), by a block of
+// The same for rows m0 .. m0 + nrows - 1 at once (at most 32 rows), by a block of
 // 32 warps: 32 / nrows warps share a row, each lane takes every 32nd of its
 // warp's tiles and the warp merges by shuffles, then one thread a row merges
 // the warps in order.  out[i] holds row i when the call returns.  (One row
 // after the other through a block-wide tree cost about 2.5 us a row.)
+// Rows nrows .. nrows + nrows2 - 1 are rows m2 .. of stats2 (row pitch m_cap2).
 constexpr int kRowWarps = 32;
 template <bool kLse>
 __device__ void reduce_rows(const float4* stats, const int2* stats_i, int w_tiles, int m_cap, int m0, int nrows,
-                            float T, RowRed* part, RowRed* out) {
+                            const float4* stats2, int m_cap2, int m2, int nrows2, float T, RowRed* part, RowRed* out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rows1 = nrows;
+  nrows += nrows2;
   const int per = kRowWarps / nrows;  // warps a row
   if (warp < per * nrows) {
-    const int m = m0 + warp / per;
+    const int row = warp / per;
+    const bool second = row >= rows1;
+    const int m = second ? m2 + row - rows1 : m0 + row;
+    if (second) { stats = stats2; m_cap = m_cap2; }
     RowRed r{-INFINITY, INT_MAX, 0.f, -INFINITY, INT_MAX};
 #pragma unroll 4
     for (int t = (warp % per) * 32 + lane; t < w_tiles; t += 32 * per) {
@@ -353,7 +374,7 @@ __device__ void reduce_rows(const float4* stats, const int2* stats_i, int w_tile
 __global__ void __launch_bounds__(256) select_kernel(const __grid_constant__ SelectArgs a) {
   pdl_wait();
   pdl_trigger();
-  __shared__ RowRed sred[256];
+  __shared__ RowRed sred[8];
   const float T = a.call->temp;
   const bool sample = a.call->sample != 0;
   int b, i = 0, m;
@@ -439,7 +460,8 @@ __global__ void __launch_bounds__(32 * kRowWarps) accept_greedy_kernel(const __g
   __shared__ RowRed s_part[kRowWarps], s_row[17];
   __shared__ int s_arg[17];
   const int b = blockIdx.x;
-  reduce_rows<false>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, 1.0f, s_part, s_row);
+  reduce_rows<false>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, nullptr, 0, 0, 0, 1.0f, s_part,
+                     s_row);
   if ((int)threadIdx.x <= a.K) s_arg[threadIdx.x] = s_row[threadIdx.x].arg;
   __syncthreads();
   if (threadIdx.x != 0) return;
@@ -465,36 +487,44 @@ void launch_accept_greedy(const AcceptArgs& a, cudaStream_t s, bool pdl) {
 __global__ void __launch_bounds__(32 * kRowWarps) accept_test_kernel(const __grid_constant__ AcceptArgs a) {
   pdl_wait();
   pdl_trigger();
-  __shared__ RowRed s_part[kRowWarps], s_row[17], s_drow[16];
+  __shared__ RowRed s_part[kRowWarps], s_row[kRowWarps];
   __shared__ float2 s_norm[17], s_dnorm[16];
-  const int b = blockIdx.x;
+  __shared__ int s_ok[16];  // candidate i's test: 1 accepted, 0 rejected, -1 outside the vocabulary
+  const int b = blockIdx.x, tid = threadIdx.x;
   const float T = a.call.temp;
-  reduce_rows<true>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, T, s_part, s_row);
-  if (a.dstats && a.K > 0)
-    reduce_rows<true>(a.dstats, nullptr, a.w_tiles, a.d_m_cap, b * a.K, a.K, T, s_part, s_drow);
-  if ((int)threadIdx.x <= a.K) s_norm[threadIdx.x] = make_float2(s_row[threadIdx.x].mx, s_row[threadIdx.x].se);
-  if ((int)threadIdx.x < a.K)
-    s_dnorm[threadIdx.x] = a.dstats ? make_float2(s_drow[threadIdx.x].mx, s_drow[threadIdx.x].se)
-                                    : a.st.dnorm[b * a.st.kmax + threadIdx.x];
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  int j = a.K;
-  for (int i = 0; i < a.K; ++i) {
-    const int di = a.st.d[b * a.st.kmax + i];
-    if (di < 0 || di >= a.vocab) {
-      // a candidate outside the vocabulary has no probability: rejected
-      if (a.status) set_status(a.status, ST_BAD_TOKEN);
-      j = i;
-      break;
+  // what the tests read besides the normalisers, requested before them
+  int di = -1;
+  float yv = 0.f, zv = 0.f;
+  if (tid < a.K) {
+    di = a.st.d[b * a.st.kmax + tid];
+    if (di >= 0 && di < a.vocab) {
+      yv = a.logits[((size_t)b * (a.K + 1) + tid) * a.vocab + di];
+      zv = a.dlogits[((size_t)b * a.K + tid) * a.vocab + di];
     }
-    const float yv = a.logits[((size_t)b * (a.K + 1) + i) * a.vocab + di];
-    const float p = expf(yv / T - s_norm[i].x / T) / s_norm[i].y;
-    const float2 zn = s_dnorm[i];
-    const float zv = a.dlogits[((size_t)b * a.K + i) * a.vocab + di];
-    const float q = expf(zv / T - zn.x / T) / zn.y;
-    const float u = uniform01(philox_word(a.call.seed, STREAM_ACCEPT, a.call.step, (uint32_t)b, (uint32_t)i, 0u));
-    if (!(u * q < p)) { j = i; break; }
   }
+  reduce_rows<true>(a.stats, a.stats_i, a.w_tiles, a.m_cap, b * (a.K + 1), a.K + 1, a.dstats, a.d_m_cap, b * a.K,
+                    a.dstats ? a.K : 0, T, s_part, s_row);
+  if (tid <= a.K) s_norm[tid] = make_float2(s_row[tid].mx, s_row[tid].se);
+  if (tid < a.K) {
+    const float2 yn = make_float2(s_row[tid].mx, s_row[tid].se);
+    const float2 zn = a.dstats ? make_float2(s_row[a.K + 1 + tid].mx, s_row[a.K + 1 + tid].se)
+                               : a.st.dnorm[b * a.st.kmax + tid];
+    s_dnorm[tid] = zn;
+    // a candidate outside the vocabulary has no probability: rejected
+    int ok = -1;
+    if (di >= 0 && di < a.vocab) {
+      const float p = expf(yv / T - yn.x / T) / yn.y;
+      const float q = expf(zv / T - zn.x / T) / zn.y;
+      const float u = uniform01(philox_word(a.call.seed, STREAM_ACCEPT, a.call.step, (uint32_t)b, (uint32_t)tid, 0u));
+      ok = u * q < p ? 1 : 0;
+    }
+    s_ok[tid] = ok;
+  }
+  __syncthreads();
+  if (tid != 0) return;
+  int j = 0;
+  while (j < a.K && s_ok[j] == 1) ++j;
+  if (j < a.K && s_ok[j] < 0 && a.status) set_status(a.status, ST_BAD_TOKEN);
   a.st.samp_a[b] = j;
   const float2 zn = j < a.K ? s_dnorm[j] : make_float2(0.f, 1.f);
   a.st.samp_norm[b] = make_float4(s_norm[j].x, s_norm[j].y, zn.x, zn.y);
@@ -504,11 +534,26 @@ __global__ void __launch_bounds__(32 * kRowWarps) accept_test_kernel(const __gri
 // from max(0, p_j - q_j) at the first rejection j, or from p_K; split over
 // kResampleSplit blocks per sequence, the last one merges in block order
 // and commits.
-__global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ AcceptArgs a) {
+constexpr int kResampleThreads = 512;
+// (value, index) maximum over the block, in s_v[0] and s_i[0]
+__device__ __forceinline__ void block_argmax(float v, int i, float* s_v, int* s_i) {
+  warp_argmax(v, i);
+  __syncthreads();  // s_v and s_i may still be read
+  if ((threadIdx.x & 31) == 0) { s_v[threadIdx.x >> 5] = v; s_i[threadIdx.x >> 5] = i; }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    v = threadIdx.x < kResampleThreads / 32 ? s_v[threadIdx.x] : -INFINITY;
+    i = threadIdx.x < kResampleThreads / 32 ? s_i[threadIdx.x] : INT_MAX;
+    warp_argmax(v, i);
+    if (threadIdx.x == 0) { s_v[0] = v; s_i[0] = i; }
+  }
+  __syncthreads();
+}
+__global__ void __launch_bounds__(kResampleThreads) resample_kernel(const __grid_constant__ AcceptArgs a) {
   pdl_wait();
   pdl_trigger();
-  __shared__ float s_v[256];
-  __shared__ int s_i[256];
+  __shared__ float s_v[kResampleThreads / 32];
+  __shared__ int s_i[kResampleThreads / 32];
   __shared__ int s_last;
   const int b = blockIdx.x / kResampleSplit, part = blockIdx.x % kResampleSplit;
   const float T = a.call.temp;
@@ -527,10 +572,9 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
   const uint64_t seed = a.call.seed;
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32), step = (uint32_t)a.call.step;
   const float cy = nm.x / T, cz = nm.z / T;
+  const bool unit = T == 1.f;  // no divisions
   for (int blk0 = v0 / 4; 4 * blk0 < v1; blk0 += blockDim.x) {
     const int blk = blk0 + threadIdx.x;
-    const U4 pw = philox4x32_10(U4{(uint32_t)blk, (uint32_t)STREAM_BONUS << 16, (uint32_t)b, step}, k0, k1);
-    const uint32_t wd[4] = {pw.x, pw.y, pw.z, pw.w};
     float yv[4], zv[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -539,6 +583,8 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
       yv[e] = in ? y[v] : 0.f;
       zv[e] = in && z ? z[v] : 0.f;
     }
+    const U4 pw = philox4x32_10(U4{(uint32_t)blk, (uint32_t)STREAM_BONUS << 16, (uint32_t)b, step}, k0, k1);
+    const uint32_t wd[4] = {pw.x, pw.y, pw.z, pw.w};
     const float wbest = warp_max(best);
     const float inv_best = expf(-wbest);
 #pragma unroll
@@ -547,31 +593,19 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
       if (v < v0 || v >= v1) continue;
       const float t = 1.0f - uniform_open01(wd[e]);  // exact
       if (z) {
-        const float p = expf(yv[e] / T - cy) / nm.y;
-        const float q = expf(zv[e] / T - cz) / nm.w;
+        const float p = expf((unit ? yv[e] : yv[e] / T) - cy) / nm.y;
+        const float q = expf((unit ? zv[e] : zv[e] / T) - cz) / nm.w;
         const float w = fmaxf(p - q, 0.f);
         if (w > 0.f && t > w * inv_best * 1.0001f) continue;
         argmax_merge(best, bi, w > 0.f ? logf(w) + gumbel(wd[e]) : -INFINITY, v);
       } else {
-        const float x = yv[e] / T;
+        const float x = unit ? yv[e] : yv[e] / T;
         if (t > expf(x - wbest) * 1.0001f) continue;
         argmax_merge(best, bi, x + gumbel(wd[e]), v);
       }
     }
   }
-  s_v[threadIdx.x] = best;
-  s_i[threadIdx.x] = bi;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) {
-      float v = s_v[threadIdx.x];
-      int i = s_i[threadIdx.x];
-      argmax_merge(v, i, s_v[threadIdx.x + w], s_i[threadIdx.x + w]);
-      s_v[threadIdx.x] = v;
-      s_i[threadIdx.x] = i;
-    }
-    __syncthreads();
-  }
+  block_argmax(best, bi, s_v, s_i);
   if (threadIdx.x == 0) {
     a.st.samp_part[b * kResampleSplit + part] = make_float2(s_v[0], __int_as_float(s_i[0]));
     __threadfence();
@@ -581,16 +615,17 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  float gbest = -INFINITY;
-  int gi = INT_MAX;
-  if (threadIdx.x == 0) {
-    for (int p = 0; p < kResampleSplit; ++p) {
-      const float2 pv = __ldcg(&a.st.samp_part[b * kResampleSplit + p]);
-      argmax_merge(gbest, gi, pv.x, __float_as_int(pv.y));
+  if (threadIdx.x < 32) {
+    // kResampleSplit partial draws, a lane each
+    const float2 pv = __ldcg(&a.st.samp_part[b * kResampleSplit + threadIdx.x]);
+    float gbest = pv.x;
+    int gi = __float_as_int(pv.y);
+    warp_argmax(gbest, gi);
+    if (threadIdx.x == 0) {
+      a.st.samp_cnt[b] = 0;
+      s_i[0] = gi;
+      s_v[0] = gbest;
     }
-    a.st.samp_cnt[b] = 0;
-    s_i[0] = gi;
-    s_v[0] = gbest;
   }
   __syncthreads();
   if (s_v[0] == -INFINITY) {
@@ -602,20 +637,7 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
       const float p = expf(y[v] / T - nm.x / T) / nm.y;
       argmax_merge(bb, bj, logf(p) + g, v);
     }
-    __syncthreads();
-    s_v[threadIdx.x] = bb;
-    s_i[threadIdx.x] = bj;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-      if ((int)threadIdx.x < w) {
-        float v = s_v[threadIdx.x];
-        int i = s_i[threadIdx.x];
-        argmax_merge(v, i, s_v[threadIdx.x + w], s_i[threadIdx.x + w]);
-        s_v[threadIdx.x] = v;
-        s_i[threadIdx.x] = i;
-      }
-      __syncthreads();
-    }
+    block_argmax(bb, bj, s_v, s_i);
   }
   if (threadIdx.x != 0) return;
   int em[17];
@@ -626,7 +648,8 @@ __global__ void __launch_bounds__(256) resample_kernel(const __grid_constant__ A
 
 void launch_accept_sample(const AcceptArgs& a, cudaStream_t s, bool pdl) {
   PARD_LAUNCH(accept_test_kernel, a.batch, 32 * kRowWarps, 0, s, pdl, a);
-  PARD_LAUNCH(resample_kernel, a.batch * kResampleSplit, 256, 0, s, true, a);
+  static_assert(kResampleSplit == 32, "a lane per partial draw");
+  PARD_LAUNCH(resample_kernel, a.batch * kResampleSplit, kResampleThreads, 0, s, true, a);
 }
 
 // Tile statistics of given logits rows (same layout as the LM-head
@@ -694,21 +717,22 @@ void launch_row_stats(const float* logits, int rows, int vocab, int w_tiles, int
               rows_per_seq > 0 ? rows_per_seq : 1, stats, stats_i);
 }
 
-// Statistics of given logits rows in tiles of kGivenTile entries (max,
-// argmax, and when sampling the sum of exp((x - max)/T)): block (t, m) takes
-// tile t of row m, the target's rows first; block (0, 0) also resets the
-// acceptance state.  HBM-bound: every logit is
-// read once, 16 bytes a load, four loads in flight a thread (batch 16, K = 6:
-// 107 MB; the whole sampled acceptance 92 us, 231 us with one 512-byte tile a
-// block, three block reductions each and one row after the other after it; the
-// greedy one at batch 1, K = 8: 9.7 us, 51.7 before).
+// Statistics of given logits rows in tiles of kGivenTile entries (the max, and
+// the argmax or, when sampling, the sum of exp((x - max)/T)): a warp takes a
+// tile, four tiles a block, the target's rows first; block (0, 0) also resets
+// the acceptance state.  Every logit is read once, 16 loads of 16 bytes in
+// flight a lane, and no block reduction follows (batch 16, K = 6: 107 MB).
+// The whole sampled acceptance takes 45 us, 231 us with one 512-byte
+// tile a block, three block reductions each and one row after the other after
+// it; the greedy one at batch 1, K = 8: 9.5 us, 51.7 before.
+template <bool kSample>  // greedy acceptance reads the argmax only, sampled the maximum and the sum
 __global__ void __launch_bounds__(128) given_stats_kernel(const __grid_constant__ GivenArgs a) {
   pdl_trigger();
-  const int t = blockIdx.x, tid = threadIdx.x, lane = tid & 31;
+  const int tid = threadIdx.x, lane = tid & 31, t = blockIdx.x * 4 + (tid >> 5);
   const bool target = (int)blockIdx.y < a.rows_t;
   const int m = target ? blockIdx.y : blockIdx.y - a.rows_t;
   const float* row = (target ? a.y : a.z) + (size_t)m * a.vocab;
-  if (t == 0 && blockIdx.y == 0) {
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
     if (tid < a.batch) {
       a.st.n[tid] = 1;
       a.st.pend_cnt[tid] = 1;
@@ -719,58 +743,56 @@ __global__ void __launch_bounds__(128) given_stats_kernel(const __grid_constant_
     }
     for (int i = tid; i < a.batch * a.K; i += 128) a.st.d[i] = a.d[i];
   }
-  float x[16];
-  int v[4];
+  if (t >= a.tiles) return;
+  // lane's entries: 16 float4s, 512 contiguous bytes a warp and load
+  float x[64];
+  const int v0 = t * kGivenTile + lane * 4;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    v[q] = t * kGivenTile + q * 512 + tid * 4;
+  for (int q = 0; q < 16; ++q) {
+    const int v = v0 + q * 128;
     float4 f = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    if (v[q] < a.vocab) {  // vocab is a multiple of 8: all four entries or none
-      if (a.vec) f = __ldcs(reinterpret_cast<const float4*>(row + v[q]));
-      else f = make_float4(row[v[q]], row[v[q] + 1], row[v[q] + 2], row[v[q] + 3]);
+    if (v < a.vocab) {  // vocab is a multiple of 8: all four entries or none
+      if (a.vec) f = __ldcs(reinterpret_cast<const float4*>(row + v));
+      else f = make_float4(row[v], row[v + 1], row[v + 2], row[v + 3]);
     }
     x[4 * q] = f.x; x[4 * q + 1] = f.y; x[4 * q + 2] = f.z; x[4 * q + 3] = f.w;
   }
-  float mv = -INFINITY;
+  float mv = -INFINITY, se = 0.f;
   int mi = INT_MAX;
 #pragma unroll
-  for (int i = 0; i < 16; ++i)
-    if (v[i / 4] < a.vocab) argmax_merge(mv, mi, x[i], v[i / 4] + (i & 3));
-  float se = 0.f;
+  for (int i = 0; i < 64; ++i) {
+    const int v = v0 + (i >> 2) * 128 + (i & 3);
+    if (kSample) mv = fmaxf(mv, x[i]);  // past the vocabulary: -infinity
+    else if (v < a.vocab) argmax_merge(mv, mi, x[i], v);
+  }
   const float T = a.call.temp;
-  if (a.sample && mv != -INFINITY) {
-    const float c = mv / T;
+  if (kSample) {
+    mv = warp_max(mv);
+    if (mv != -INFINITY) {  // past the vocabulary: exp(-infinity) = 0
+      if (T == 1.f) {       // no divisions
 #pragma unroll
-    for (int i = 0; i < 16; ++i) se += v[i / 4] < a.vocab ? expf(x[i] / T - c) : 0.f;
-  }
-  auto merge = [&](float m2, int i2, float s2) {
-    if (a.sample) {
-      float mm = mv;
-      merge_lse(mm, se, m2, s2, T);
+        for (int i = 0; i < 64; ++i) se += expf(x[i] - mv);
+      } else {
+        const float c = mv / T;
+#pragma unroll
+        for (int i = 0; i < 64; ++i) se += expf(x[i] / T - c);
+      }
     }
-    argmax_merge(mv, mi, m2, i2);
-  };
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const float m2 = __shfl_xor_sync(0xffffffffu, mv, o), s2 = __shfl_xor_sync(0xffffffffu, se, o);
-    const int i2 = __shfl_xor_sync(0xffffffffu, mi, o);
-    merge(m2, i2, s2);
+    se = warp_sum(se);
+  } else {
+    warp_argmax(mv, mi);
   }
-  __shared__ float s_m[4], s_s[4];
-  __shared__ int s_i[4];
-  if (lane == 0) { s_m[tid >> 5] = mv; s_s[tid >> 5] = se; s_i[tid >> 5] = mi; }
-  __syncthreads();
-  if (tid == 0) {
-    for (int w = 1; w < 4; ++w) merge(s_m[w], s_i[w], s_s[w]);
+  if (lane == 0) {
     const size_t at = (size_t)t * (target ? a.m_cap_t : a.m_cap_d) + m;
     (target ? a.stats_t : a.stats_d)[at] = make_float4(mv, se, -INFINITY, 0.f);
-    if (target) a.stats_it[at] = make_int2(mi, -1);
+    if (!kSample) a.stats_it[at] = make_int2(mi, -1);
   }
 }
 
 void launch_given_stats(const GivenArgs& a, cudaStream_t s) {
-  PARD_LAUNCH(given_stats_kernel, dim3((a.vocab + kGivenTile - 1) / kGivenTile, a.rows_t + a.rows_d), 128, 0, s, false,
-              a);
+  const dim3 grid((a.tiles + 3) / 4, a.rows_t + a.rows_d);
+  if (a.sample) PARD_LAUNCH(given_stats_kernel<true>, grid, 128, 0, s, false, a);
+  else PARD_LAUNCH(given_stats_kernel<false>, grid, 128, 0, s, false, a);
 }
 
 __global__ void set_call_kernel(CallArgs* dst, CallArgs v) {

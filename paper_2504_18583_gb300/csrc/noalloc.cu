@@ -134,6 +134,7 @@ extern "C" pard_status pard_accept_noalloc(const float* d_target_logits, const f
     memset(&g, 0, sizeof(g));
     g.y = d_target_logits; g.z = d_draft_logits;
     g.rows_t = batch * (K + 1); g.rows_d = sample ? batch * K : 0;
+    g.tiles = tiles;
     g.m_cap_t = kNaRowsT; g.m_cap_d = kNaRowsD; g.vocab = vocab;
     g.vec = ((reinterpret_cast<uintptr_t>(d_target_logits) | (sample ? reinterpret_cast<uintptr_t>(d_draft_logits) : 0)) &
              15) == 0;
