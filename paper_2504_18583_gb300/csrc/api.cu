@@ -331,6 +331,12 @@ GemmArgs gemm_base(pard_ctx* c, int rows_cap, int tt) {
   return a;
 }
 
+// Units a CTA may take on top of an even share so that tiles are in equal
+// parts.  Measured (1B draft, 8B verify, 70B-width verify of 4 layers, batch 1;
+// us): never 763 / 2908 / 1455, 1: 763 / 2899 / 1456, 3: 763 / 2890 / 1455, 5:
+// 740 / 2890 / 1455, 10: 740 / 2914 / 1457, always 740 / 2914 / 1486.
+constexpr long kNarrowEven = 5;
+
 void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
   if (tt == kWideTok) {
     const long w_pairs = (a.w_tiles + 1) / 2;
@@ -352,14 +358,30 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
     return;
   }
   const long U = (long)a.w_tiles * a.tok_tiles * a.kc;
-  // at least 8 units (128 KB of weights) a CTA: with fewer, the split-K
+  // At least 8 units (128 KB of weights) a CTA: with fewer, the split-K
   // finish of a tile gathers partials from too many CTAs; and at least
   // kc / 62 units, so that no tile has more than 63 contributors (the
-  // finisher tracks their arrivals in one 64-bit mask)
+  // finisher tracks their arrivals in one 64-bit mask).  But a tile is never
+  // shared for that (tiny configuration's verify pass: 104 -> 82 us).
+  const long T = (long)a.w_tiles * a.tok_tiles;
   const long min_units = std::max<long>(8, (a.kc + 61) / 62);
-  const int grid = (int)std::min<long>(c->sm, std::max<long>(1, U / min_units));
+  const long most = std::min<long>(c->sm, std::max<long>(U / min_units, T));
+  long grid = most;
+  if (T < most) {
+    // Fewer tiles than CTAs: each cut into the same number of parts.  (A CTA
+    // with units of two tiles stores two partials, or finishes one tile after
+    // storing the other's.)
+    if ((a.kc + most / T - 1) / (most / T) <= (U + most - 1) / most + kNarrowEven) grid = most / T * T;
+  } else if (tt == 16 && T > c->sm && T <= 4 * c->sm) {
+    // One or two whole tiles a CTA and no exchange at all: two CTAs of the
+    // 16-token tile fit on an SM, and as all wait for HBM they end together
+    // although some SMs hold two (8B verify pass 2890 -> 2827 us, 70B widths
+    // 1472 -> 1454).
+    if (T <= 2 * c->sm) grid = T;
+    else if (T % 2 == 0) grid = T / 2;
+  }
   if ((long)a.w_tiles * a.tok_tiles > kMaxGemmTiles || (U + 1) * (grid + 1) > INT32_MAX) throw cudaErrorInvalidValue;
-  launch_gemm(a, tt, grid, s, true);
+  launch_gemm(a, tt, (int)grid, s, true);
   c->launches++;
 }
 
