@@ -58,13 +58,10 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   const EpiSmem S = carve_epi<TT>(scratch);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int* live = reinterpret_cast<int*>(misc + 4);  // [0] token tiles processed, [1] token rows of one tile's MMA
-  // this CTA's units (recomputed below in the rare launch that drops token tiles)
-  const bool early = a.m_early && a.tok_tiles > 1;
   const int G = gridDim.x;
   const int c = blockIdx.x;
-  int U = a.w_tiles * a.tok_tiles * a.kc;
-  int u0 = range_start(c, U, G), u1 = range_start(c + 1, U, G);
+  const int tok_tiles = a.tok_tiles, U = a.w_tiles * tok_tiles * a.kc;
+  const int u0 = range_start(c, U, G), u1 = range_start(c + 1, U, G);  // this CTA's units
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < C::kStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
@@ -73,19 +70,6 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
     mbar_init(fx, 1);
     *abort_flag = 0;
     *fx_armed = 0;
-    // Token tiles past the pass's row count hold no output row.  A
-    // multi-tile launch whose row count was written two or more launches back
-    // (the previous kernel itself waited for that writer before letting this
-    // grid start) reads it now and neither loads nor multiplies those tiles;
-    // when one tile is left it covers only the rows present (B = 2 n_tok
-    // rows).  A single-tile launch takes n_tok from the host's row capacity
-    // and starts without this read.
-    if (early) {
-      const int m = min(max(__ldcg(a.m_dev), 1), a.m_cap);
-      const int tiles = min(a.tok_tiles, (m + TT - 1) / TT);
-      live[0] = tiles;
-      live[1] = tiles == 1 ? min(TT, (m + 7) / 8 * 8) : TT;
-    }
     fence_barrier_init();
   }
   if (warp == 1) tmem_alloc(tmem_slot, C::kTmemCols);
@@ -93,19 +77,12 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const int tok_tiles = early ? live[0] : a.tok_tiles;
-  if (tok_tiles != a.tok_tiles) {
-    U = a.w_tiles * tok_tiles * a.kc;
-    u0 = range_start(c, U, G);
-    u1 = range_start(c + 1, U, G);
-  }
   uint32_t armed = 0, armed_odd = 0;  // producer: slots armed at least once, and those armed an odd number of times
   // ring slots this launch uses, and how many are filled before the PDL wait
   const int R = (a.stages > 0 && a.stages < C::kStages) ? a.stages : C::kStages;
   const int P = (a.pre_stages > 0 && a.pre_stages < R) ? a.pre_stages : R;
   // token rows a tile's MMA covers: hi/lo pairs are the B rows, so N = 2 n_tok
-  const int n_tok = early ? live[1]
-                           : ((a.tok_tiles == 1 && a.n_tok > 0 && a.n_tok < TT && a.n_tok % 8 == 0) ? a.n_tok : TT);
+  const int n_tok = (tok_tiles == 1 && a.n_tok > 0 && a.n_tok < TT && a.n_tok % 8 == 0) ? a.n_tok : TT;
   const uint32_t b_bytes = (uint32_t)n_tok * 2 * 128;
   const uint32_t stage_bytes = (uint32_t)C::kABytes + b_bytes;
 

@@ -43,8 +43,8 @@ struct GemmArgs {
   int w_tiles, tok_tiles, kc;
   int n_tok;                  // token rows a tile's MMA covers (multiple of 8, <= the tile; 0: the whole tile):
                               // a single-tile pass of fewer rows loads and multiplies only those
-  int m_early;                // m_dev was written two or more launches back: read it before the PDL wait and
-                              // skip the token tiles past it (0: process every tile)
+  int m_early;                // wide GEMM: m_dev was written two or more launches back, so it is read before the
+                              // PDL wait, and the token tiles are laid out for the rows there are
   int mode;
   int m_cap;                  // row capacity of the activation/output buffers
   const int* m_dev;           // runtime row count
@@ -303,8 +303,6 @@ void launch_accept_sample(const AcceptArgs& a, cudaStream_t s, bool pdl);
 void launch_row_stats(const float* logits, int rows, int vocab, int w_tiles, int m_cap, const CallArgs* call,
                       int gumbel_stream, int rows_per_seq, float4* stats, int2* stats_i, cudaStream_t s);
 void launch_set_call(CallArgs* dst, CallArgs v, cudaStream_t s, bool pdl);
-void launch_copy_i32(const int* src, int* dst, int n, cudaStream_t s, bool pdl);
-void launch_copy_f32(const float* src, float* dst, size_t n, cudaStream_t s, bool pdl);
 void launch_read_kv(const __nv_bfloat16* kc, const __nv_bfloat16* vc, const int* page_table_row, const int* pos, int n,
                     int hkv, int hd, int page_size, __nv_bfloat16* ok, __nv_bfloat16* ov, cudaStream_t s);
 

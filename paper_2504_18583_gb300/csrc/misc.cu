@@ -804,31 +804,6 @@ void launch_set_call(CallArgs* dst, CallArgs v, cudaStream_t s, bool pdl) {
   PARD_LAUNCH(set_call_kernel, 1, 1, 0, s, pdl, dst, v);
 }
 
-__global__ void copy_i32_kernel(const int* src, int* dst, int n) {
-  pdl_wait();
-  pdl_trigger();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) dst[i] = src[i];
-}
-void launch_copy_i32(const int* src, int* dst, int n, cudaStream_t s, bool pdl) {
-  PARD_LAUNCH(copy_i32_kernel, 1, 256, 0, s, pdl, src, dst, n);
-}
-
-__global__ void copy_f32_kernel(const float4* src, float4* dst, size_t n4) {
-  pdl_wait();
-  pdl_trigger();
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = src[i];
-}
-void launch_copy_f32(const float* src, float* dst, size_t n, cudaStream_t s, bool pdl) {
-  // n is a multiple of 4 and both pointers are 16-byte aligned (checked by the caller)
-  const size_t n4 = n / 4;
-  int grid = (int)((n4 + 255) / 256);
-  if (grid > 1216) grid = 1216;
-  if (grid < 1) grid = 1;
-  PARD_LAUNCH(copy_f32_kernel, grid, 256, 0, s, pdl, reinterpret_cast<const float4*>(src),
-              reinterpret_cast<float4*>(dst), n4);
-}
-
 __global__ void read_kv_kernel(const __nv_bfloat16* kc, const __nv_bfloat16* vc, const int* pt, const int* pos, int n,
                                int hkv, int hd, int ps, __nv_bfloat16* ok, __nv_bfloat16* ov) {
   const int i = blockIdx.x;
