@@ -17,7 +17,7 @@
 // (4096 bins for at most 4096 keys: the words are uniform, so the bin the
 // threshold falls into holds a key or two) and a rank count among that bin's
 // members alone, instead of every candidate counting over the whole subtask
-// (2048 rows, K = 8: 24.6 us, 971 us with the O(n^2) count on one SM).  Thread t
+// (2048 rows, K = 8: 18.8 us, 971 us with the O(n^2) count on one SM).  Thread t
 // holds rows 4t .. 4t+3, the four words of one Philox block.
 #include "common.cuh"
 #include "internal.h"
@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(kCodThreads) cod_kernel(int N, int K, double r
   __shared__ uint16_t s_lrow[kCodMaxN];
   __shared__ uint32_t s_keep[kCodThreads];       // the previous subtask's flags, one byte a row
   __shared__ int s_warp[kCodThreads / 32];
+  __shared__ int s_n[64];
   __shared__ int s_bin, s_need, s_total, s_members;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int* hist = reinterpret_cast<int*>(s_hist);
@@ -43,12 +44,16 @@ __global__ void __launch_bounds__(kCodThreads) cod_kernel(int N, int K, double r
   const bool vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(keep) & 15) == 0;
   s_hist[tid] = make_int4(0, 0, 0, 0);
   if (tid == 0) counts[0] = N;
-  double g = 1.0;
+  // rows kept by each subtask, a thread a subtask: the double-precision unit is
+  // too narrow for 32 warps to compute them in every subtask
+  if (tid < K - 1) {
+    double g = 1.0;
+    for (int i = 0; i <= tid; ++i) g *= r;
+    s_n[tid] = (int)floor((double)N * (g > r_min ? g : r_min) + 0.5);
+  }
   __syncthreads();
   for (int k = 2; k <= K; ++k) {
-    g *= r;
-    const double gam = g > r_min ? g : r_min;
-    const int n = (int)floor((double)N * gam + 0.5);
+    const int n = s_n[k - 2];
     // flags of rows j0 - 1 .. j0 + 2 of subtask k - 1, a byte each
     uint32_t prev = 0x01010101u;
     if (k > 2) prev = (s_keep[tid] << 8) | (tid > 0 ? s_keep[tid - 1] >> 24 : 0u);
