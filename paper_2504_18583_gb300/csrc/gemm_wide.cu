@@ -19,12 +19,21 @@
 // partials in pair order (deterministic).  (One finisher per tile gathers all
 // partials of up to 128 KB each on one SM, which took longer than the
 // multiplication.)  A pair waits for the others only after its last unit is
-// multiplied and stored, so no wait closes a circle.
+// multiplied and stored, and not for long: it gives its share up to the last
+// one to arrive, so that no CTA holds its SM for CTAs that have none yet.
 //
 // Roles per CTA: warp 0 streams, counting both CTAs' bytes on rank 0's
 // barriers (TMA tensor copies can do that; the packed operands are tensors of
 // 128-byte rows to them), warp 1 of rank 0 issues the MMAs, warps 2-5 and 6-9
 // are two epilogue groups that take alternate chunks.
+//
+// Measured (one layer's launches, serialised, us; before: 64-token tiles, and a
+// 128-token tile for gate/up and LM head, on single CTAs): 8B widths, 112 rows:
+// QKV 36 -> 24, O 30 -> 23, gate/up 62 -> 52 (34 at the HBM rate), down 52 -> 36,
+// LM head 236 -> 183; 512 rows, first form with even shares only: 82 -> 58,
+// 57 -> 50, 197 -> 148, 138 -> 91.  The main loop runs at 1.14k clocks per step of
+// 256 x 256 x 64 (hi and lo: 2 x 8.4 MFLOP a CTA) or at 7 TB/s of weights; what
+// is left is each launch's start and its tail (partials, arrival, shares).
 #include "gemm_core.cuh"
 
 namespace pard {
@@ -85,6 +94,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
   int* bcast = reinterpret_cast<int*>(misc + 2);
   volatile int* fx_armed = reinterpret_cast<volatile int*>(misc + 3);  // rounds of copies issued
   int* live = reinterpret_cast<int*>(misc + 4);  // [0] token tiles, [1] tokens a tile
+  uint32_t* extra = misc + 6;                    // [2] shares given up by others that fall to this CTA, per split tile
   float* rs = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(misc) + kWideMiscBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -328,9 +338,15 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
     // A split tile this pair has stored its partial of, and its share of it:
     // contributor i of n finishes chunks [ceil(i nch / n), ceil((i + 1) nch / n))
     struct Share {
-      int t, w_tile, tok_base, cf, n, readers, c0, c1;
+      int t, w_tile, tok_base, cf, n, nch, i, c0, c1;
     };
-    Share sh0{0, 0, 0, 0, 1, 0, 0, 0}, sh1{0, 0, 0, 0, 1, 0, 0, 0};
+    Share sh0{0, 0, 0, 0, 1, 0, 0, 0, 0}, sh1{0, 0, 0, 0, 1, 0, 0, 0, 0};
+    bool settled = false;  // it is known which shares are this CTA's
+    uint32_t todo0 = 0, todo1 = 0;  // contributors whose shares it takes besides its own
+    auto range_of = [](Share& h, int i) {
+      h.c0 = (i * h.nch + h.n - 1) / h.n;
+      h.c1 = ((i + 1) * h.nch + h.n - 1) / h.n;
+    };
     auto mask_of = [&](int t) { return reinterpret_cast<unsigned long long*>(a.counters) + 2 * t + rank; };
     auto partial = [&](const Share& h, int k) {
       // only the tile's first contributor may begin before the tile
@@ -406,14 +422,52 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
           if (et == 0) mbar_arrive_remote(&acce[ab], 0);
           if (!last) continue;
           const int cf = owner(t * kc), n = owner((t + 1) * kc - 1) - cf + 1, i = c - cf;
-          if (et256 == 0 && nch > 0) red_release_or64(mask_of(t), 1ull << i);
-          const Share h{t, wt0, tb0, cf, n, min(n, nch), (i * nch + n - 1) / n, ((i + 1) * nch + n - 1) / n};
+          if (et256 == 0) {
+            uint32_t given = 0;
+            if (nch > 0) {
+              const unsigned long long all = contrib_bits(n), old = atom_or64(mask_of(t), 1ull << i);
+              if (((old | 1ull << i) & all) == all) given = (uint32_t)((old >> kWideContrib) & all);
+            }
+            extra[slot] = given;
+          }
+          Share h{t, wt0, tb0, cf, n, nch, i, 0, 0};
+          range_of(h, i);
           if (slot == 0) sh0 = h;
           else sh1 = h;
           continue;
         }
       } else {
-        const int rem0 = sh0.c1 - sh0.c0, rem1 = sh1.c1 - sh1.c0;
+        if (!settled) {
+          settled = true;
+          if (et256 == 0) {
+            // until all partials of the share's tile are stored, or too long:
+            // whoever finds the tile complete in its own atomic is in charge
+            auto settle = [&](const Share& h) {
+              if (h.c0 >= h.c1) return 1;
+              const unsigned long long all = contrib_bits(h.n), t0 = globaltimer();
+              while ((ld_acquire_u64(mask_of(h.t)) & all) != all)
+                if (globaltimer() - t0 > kShareWaitNs)
+                  return (atom_or64(mask_of(h.t), 1ull << (kWideContrib + h.i)) & all) == all ? 1 : 0;
+              return 1;
+            };
+            const int mine0 = settle(sh0), mine1 = settle(sh1);
+            bcast[0] = mine0 | mine1 << 1;
+          }
+          all_epi_bar();
+          if (!(bcast[0] & 1)) sh0.c0 = sh0.c1;
+          if (!(bcast[0] & 2)) sh1.c0 = sh1.c1;
+          if (sh0.nch > 0) todo0 = extra[0];
+          if (sh1.nch > 0) todo1 = extra[1];
+        }
+        while (sh0.c0 >= sh0.c1 && todo0) {
+          range_of(sh0, __ffs((int)todo0) - 1);
+          todo0 &= todo0 - 1;
+        }
+        while (sh1.c0 >= sh1.c1 && todo1) {
+          range_of(sh1, __ffs((int)todo1) - 1);
+          todo1 &= todo1 - 1;
+        }
+        const int rem0 = max(0, sh0.c1 - sh0.c0), rem1 = max(0, sh1.c1 - sh1.c0);
         if (rem0 + rem1 == 0) break;
         n0 = sh0.n; n1 = sh1.n;
         take0 = min(rem0, kRingChunks / n0);
@@ -441,52 +495,26 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
       }
       if (!from_acc) {
         if (et256 == 0) {
-          bool got = true;
           if (staged) {
-            fence_proxy_async_all();  // the ring was read by the previous round
+            // the ring was read by the previous round; the partials were
+            // written through the generic proxy, the copies read them through
+            // the async proxy
+            fence_proxy_async_all();
             *fx_armed = rounds + 1;
             mbar_arrive_expect_tx(fx, (uint32_t)(take0 * n0 + take1 * n1) * kChF * 4);
+            auto fetch = [&](const Share& h, int take, int at) {
+              for (int k = 0; k < h.n && take; ++k)
+                bulk_load(reinterpret_cast<float*>(ring) + (size_t)(at + k * take) * kChF, partial(h, k) + (size_t)h.c0 * kChF,
+                          (uint32_t)take * kChF * 4, fx);
+            };
+            fetch(sh0, take0, 0);
+            fetch(sh1, take1, base1);
           }
-          const unsigned long long all0 = take0 ? contrib_bits(n0) : 0, all1 = take1 ? contrib_bits(n1) : 0;
-          unsigned long long seen0 = 0, seen1 = 0;
-          const unsigned long long t0 = globaltimer();
-          // copies of the contributors that have arrived since the last look;
-          // the partials were written through the generic proxy, the copies
-          // read them through the async proxy
-          auto fetch = [&](const Share& h, unsigned long long all, unsigned long long& seen, int take, int at) {
-            const unsigned long long m = ld_acquire_u64(mask_of(h.t)) & all;
-            unsigned long long nw = m & ~seen;
-            if (!nw) return false;
-            fence_proxy_async();
-            while (nw && staged) {
-              const int k = __ffsll((long long)nw) - 1;
-              nw &= nw - 1;
-              bulk_load(reinterpret_cast<float*>(ring) + (size_t)(at + k * take) * kChF, partial(h, k) + (size_t)h.c0 * kChF,
-                        (uint32_t)take * kChF * 4, fx);
-            }
-            seen = m;
-            return true;
-          };
-          while (seen0 != all0 || seen1 != all1) {
-            bool any = false;
-            if (seen0 != all0) any |= fetch(sh0, all0, seen0, take0, 0);
-            if (seen1 != all1) any |= fetch(sh1, all1, seen1, take1, base1);
-            if (!any && (*abort_flag || globaltimer() - t0 > kWaitLimitNs)) {
-              got = false;
-              break;
-            }
-          }
-          if (!got) set_status(a.status, ST_TIMEOUT_EPI);
-          bcast[0] = got ? 1 : 0;
           // last round of a share: count it in the mask's upper byte (read below)
-          if (got && take0 && sh0.c0 + take0 == sh0.c1)
-            old0 = atomicAdd(mask_of(sh0.t), 1ull << kWideReadShift);
-          if (got && take1 && sh1.c0 + take1 == sh1.c1)
-            old1 = atomicAdd(mask_of(sh1.t), 1ull << kWideReadShift);
+          if (take0 && sh0.c0 + take0 == sh0.c1) old0 = atomicAdd(mask_of(sh0.t), 1ull << kWideReadShift);
+          if (take1 && sh1.c0 + take1 == sh1.c1) old1 = atomicAdd(mask_of(sh1.t), 1ull << kWideReadShift);
         }
-        all_epi_bar();
-        ok = bcast[0] != 0;
-        if (ok && staged) ok = mbar_wait(fx, (uint32_t)(rounds & 1), abort_flag);
+        ok = !staged || mbar_wait(fx, (uint32_t)(rounds & 1), abort_flag);
         if (all_epi_any(!ok)) {
           if (et256 == 0) set_status(a.status, ST_TIMEOUT_EPI);
           *abort_flag = 1;
@@ -546,13 +574,12 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         epi_bar(S.bar);
         if (et == 0) mbar_arrive_remote(&acce[ab], 0);
       } else {
-        if (sh0.c0 + take0 + (sh1.c0 + take1) < sh0.c1 + sh1.c1)
-          all_epi_bar();  // the ring is read out before the next round
+        all_epi_bar();  // the ring is read out before the next round
         if (et256 == 0) {
           // the last of the finishing CTAs clears the mask
-          if (take0 && sh0.c0 + take0 == sh0.c1 && (int)(old0 >> kWideReadShift) == sh0.readers - 1)
+          if (take0 && sh0.c0 + take0 == sh0.c1 && (int)(old0 >> kWideReadShift) == min(sh0.n, sh0.nch) - 1)
             *mask_of(sh0.t) = 0ull;
-          if (take1 && sh1.c0 + take1 == sh1.c1 && (int)(old1 >> kWideReadShift) == sh1.readers - 1)
+          if (take1 && sh1.c0 + take1 == sh1.c1 && (int)(old1 >> kWideReadShift) == min(sh1.n, sh1.nch) - 1)
             *mask_of(sh1.t) = 0ull;
         }
         sh0.c0 += take0;

@@ -231,7 +231,15 @@ constexpr int kMaxAttnSplit = 16;       // key splits (CTAs of one cluster) of o
 // Wide GEMM (gemm_wide.cu; passes of more than 64 rows): tiles of 256 weight
 // rows and at most kWideTok tokens, multiplied by a pair of CTAs.
 constexpr int kWideTok = 256;
-constexpr int kWideReadShift = 56;  // a split tile's mask word: 56 contributors, and above them its finished shares
+// A split tile's mask word: a bit per contributor that has stored its partial,
+// a bit per contributor that has given its share up, and above them the number
+// of finished shares.
+constexpr int kWideContrib = 28, kWideReadShift = 2 * kWideContrib;
+// A contributor waits this long for the others of its tile before it gives its
+// share up to the last one to arrive (usually they arrive within 10 us): every
+// CTA of a launch ends in bounded time without the others, as it must where
+// launches of two streams share the SMs and neither is wholly on them.
+constexpr unsigned long long kShareWaitNs = 100000;
 // Units of the QKV projection that one accumulator sums before the epilogue
 // adds it up in fp32 registers: the tensor cores truncate at every
 // accumulation (hi and lo parts: eight a unit), and keys and values are
@@ -272,8 +280,8 @@ struct WideSplit {
   bool tiles;  // ranges are whole tiles
 };
 __host__ __device__ inline WideSplit wide_split(int T, int kc, int max_pairs) {
-  // at least four units (64 KB of weights a CTA) a pair, and at most 56 pairs to a tile
-  const int least = kc > 4 * 54 ? (kc + 53) / 54 : 4;
+  // at least four units (64 KB of weights a CTA) a pair, and at most kWideContrib pairs to a tile
+  const int least = kc > 4 * (kWideContrib - 2) ? (kc + kWideContrib - 3) / (kWideContrib - 2) : 4;
   const int most = T * kc / least < 1 ? 1 : (T * kc / least < max_pairs ? T * kc / least : max_pairs);
   const int even = (T * kc + most - 1) / most;
   if (T >= most) return {most, (T + most - 1) / most * kc <= even + kWideExchange};
