@@ -19,8 +19,8 @@
 // partials in pair order (deterministic).  (One finisher per tile gathers all
 // partials of up to 128 KB each on one SM, which took longer than the
 // multiplication.)  A pair waits for the others only after its last unit is
-// multiplied and stored, and not for long: it gives its share up to the last
-// one to arrive, so that no CTA holds its SM for CTAs that have none yet.
+// multiplied and stored, and not for long: it gives its share up to one
+// that arrives later, so that no CTA holds its SM for CTAs that have none yet.
 //
 // Roles per CTA: warp 0 streams, counting both CTAs' bytes on rank 0's
 // barriers (TMA tensor copies can do that; the packed operands are tensors of
@@ -76,6 +76,20 @@ __device__ __forceinline__ void load_acc(uint32_t taddr, float (&v)[kEpiTok]) {
 }
 
 }  // namespace
+
+// Shares of a complete tile that were given up go to whoever takes their bits
+// out of its word.  The last contributor to arrive sees, after its own bit, all
+// bits set before that; who gives up later sees the tile complete.  Both calls
+// are rare and out of line: inlined, they lengthened every launch's tail (a
+// batch-16 draft pass: 1640 us, 1599 so; 1588 without giving up at all).
+static __device__ __noinline__ uint32_t claim_shares(unsigned long long* word, uint32_t given) {
+  return (uint32_t)(atom_and64(word, ~((unsigned long long)given << kWideContrib)) >> kWideContrib) & given;
+}
+// gives up contributor i's share; which shares are the caller's all the same
+static __device__ __noinline__ uint32_t give_share_up(unsigned long long* word, unsigned long long all, int i) {
+  const unsigned long long own = 1ull << (kWideContrib + i), w = atom_or64(word, own) | own;
+  return (w & all) == all ? claim_shares(word, (uint32_t)(w >> kWideContrib & all)) : 0u;
+}
 
 template <int MODE>
 __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid_constant__ WideArgs w) {
@@ -353,6 +367,22 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
       const int sl = k > 0 || start_of(h.cf) >= h.t * kc ? 0 : 1;
       return a.partials + ((size_t)(2 * (h.cf + k) + rank) * 2 + sl) * kTileF;
     };
+    auto claim = [&](const Share& h, unsigned long long w, int slot) {
+      const uint32_t given = (uint32_t)(w >> kWideContrib & contrib_bits(h.n));
+      if (given) extra[slot] |= claim_shares(mask_of(h.t), given);
+    };
+    auto look = [&](const Share& h, int slot) {
+      if (h.nch <= 0 || h.c0 < h.c1) return;
+      const unsigned long long all = contrib_bits(h.n), w = ld_acquire_u64(mask_of(h.t));
+      if ((w & all) == all) claim(h, w, slot);
+    };
+    auto settle = [&](int mine) {
+      settled = true;
+      if (!(mine & 1)) sh0.c0 = sh0.c1;
+      if (!(mine & 2)) sh1.c0 = sh1.c1;
+      if (sh0.nch > 0) todo0 = extra[0];
+      if (sh1.nch > 0) todo1 = extra[1];
+    };
     int seg_i = 0, rounds = 0;
     bool ok = true;
     int u = u0;
@@ -423,12 +453,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
           if (!last) continue;
           const int cf = owner(t * kc), n = owner((t + 1) * kc - 1) - cf + 1, i = c - cf;
           if (et256 == 0) {
-            uint32_t given = 0;
-            if (nch > 0) {
-              const unsigned long long all = contrib_bits(n), old = atom_or64(mask_of(t), 1ull << i);
-              if (((old | 1ull << i) & all) == all) given = (uint32_t)((old >> kWideContrib) & all);
-            }
-            extra[slot] = given;
+            if (nch > 0) red_release_or64(mask_of(t), 1ull << i);
+            extra[slot] = 0;
           }
           Share h{t, wt0, tb0, cf, n, nch, i, 0, 0};
           range_of(h, i);
@@ -437,27 +463,14 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
           continue;
         }
       } else {
-        if (!settled) {
-          settled = true;
+        // its own shares first; those that others gave up after them
+        if (!settled && sh0.c0 >= sh0.c1 && sh1.c0 >= sh1.c1) {
           if (et256 == 0) {
-            // until all partials of the share's tile are stored, or too long:
-            // whoever finds the tile complete in its own atomic is in charge
-            auto settle = [&](const Share& h) {
-              if (h.c0 >= h.c1) return 1;
-              const unsigned long long all = contrib_bits(h.n), t0 = globaltimer();
-              while ((ld_acquire_u64(mask_of(h.t)) & all) != all)
-                if (globaltimer() - t0 > kShareWaitNs)
-                  return (atom_or64(mask_of(h.t), 1ull << (kWideContrib + h.i)) & all) == all ? 1 : 0;
-              return 1;
-            };
-            const int mine0 = settle(sh0), mine1 = settle(sh1);
-            bcast[0] = mine0 | mine1 << 1;
+            look(sh0, 0);
+            look(sh1, 1);
           }
           all_epi_bar();
-          if (!(bcast[0] & 1)) sh0.c0 = sh0.c1;
-          if (!(bcast[0] & 2)) sh1.c0 = sh1.c1;
-          if (sh0.nch > 0) todo0 = extra[0];
-          if (sh1.nch > 0) todo1 = extra[1];
+          settle(3);
         }
         while (sh0.c0 >= sh0.c1 && todo0) {
           range_of(sh0, __ffs((int)todo0) - 1);
@@ -495,30 +508,77 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
       }
       if (!from_acc) {
         if (et256 == 0) {
+          uint32_t mine = 3;
+          if (staged) fence_proxy_async_all();  // the ring was read by the previous round
+          // copies of the contributors that have arrived since the last look;
+          // the partials were written through the generic proxy, the copies
+          // read them through the async proxy
+          auto fetch = [&](const Share& h, unsigned long long all, unsigned long long& seen, int take, int at, int slot) {
+            const unsigned long long w = settled ? all : ld_acquire_u64(mask_of(h.t)), m = w & all;
+            if (m == all && !settled) claim(h, w, slot);
+            unsigned long long nw = m & ~seen;
+            if (!nw) return false;
+            fence_proxy_async();
+            for (; nw && staged && take; nw &= nw - 1) {
+              const int k = __ffsll((long long)nw) - 1;
+              const uint32_t bytes = (uint32_t)take * kChF * 4;
+              mbar_expect_tx(fx, bytes);
+              bulk_load(reinterpret_cast<float*>(ring) + (size_t)(at + k * take) * kChF, partial(h, k) + (size_t)h.c0 * kChF, bytes,
+                        fx);
+            }
+            seen = m;
+            return true;
+          };
+          // (a share without room in this round is settled all the same)
+          const unsigned long long all0 = sh0.c0 < sh0.c1 ? contrib_bits(n0) : 0, all1 = sh1.c0 < sh1.c1 ? contrib_bits(n1) : 0;
+          unsigned long long seen0 = 0, seen1 = 0;
+          const unsigned long long t0 = globaltimer();
+          while (seen0 != all0 || seen1 != all1) {
+            bool any = false;
+            if (seen0 != all0) any |= fetch(sh0, all0, seen0, take0, 0, 0);
+            if (seen1 != all1) any |= fetch(sh1, all1, seen1, take1, base1, 1);
+            if (!any && globaltimer() - t0 > kShareWaitNs) {
+              // not in time: the round is done anew, without what is no longer this CTA's
+              mine = 7;
+              if (seen0 != all0) {
+                const uint32_t e = give_share_up(mask_of(sh0.t), all0, sh0.i);
+                if (!(e >> sh0.i & 1)) mine &= ~1u;
+                extra[0] |= e & ~(1u << sh0.i);
+              }
+              if (seen1 != all1) {
+                const uint32_t e = give_share_up(mask_of(sh1.t), all1, sh1.i);
+                if (!(e >> sh1.i & 1)) mine &= ~2u;
+                extra[1] |= e & ~(1u << sh1.i);
+              }
+              break;
+            }
+          }
           if (staged) {
-            // the ring was read by the previous round; the partials were
-            // written through the generic proxy, the copies read them through
-            // the async proxy
-            fence_proxy_async_all();
             *fx_armed = rounds + 1;
-            mbar_arrive_expect_tx(fx, (uint32_t)(take0 * n0 + take1 * n1) * kChF * 4);
-            auto fetch = [&](const Share& h, int take, int at) {
-              for (int k = 0; k < h.n && take; ++k)
-                bulk_load(reinterpret_cast<float*>(ring) + (size_t)(at + k * take) * kChF, partial(h, k) + (size_t)h.c0 * kChF,
-                          (uint32_t)take * kChF * 4, fx);
-            };
-            fetch(sh0, take0, 0);
-            fetch(sh1, take1, base1);
+            mbar_arrive(fx);
+          }
+          if (!settled) {
+            look(sh0, 0);
+            look(sh1, 1);
+            bcast[0] = (int)mine;
           }
           // last round of a share: count it in the mask's upper byte (read below)
-          if (take0 && sh0.c0 + take0 == sh0.c1) old0 = atomicAdd(mask_of(sh0.t), 1ull << kWideReadShift);
-          if (take1 && sh1.c0 + take1 == sh1.c1) old1 = atomicAdd(mask_of(sh1.t), 1ull << kWideReadShift);
+          if (mine == 3 && take0 && sh0.c0 + take0 == sh0.c1) old0 = atomicAdd(mask_of(sh0.t), 1ull << kWideReadShift);
+          if (mine == 3 && take1 && sh1.c0 + take1 == sh1.c1) old1 = atomicAdd(mask_of(sh1.t), 1ull << kWideReadShift);
         }
         ok = !staged || mbar_wait(fx, (uint32_t)(rounds & 1), abort_flag);
         if (all_epi_any(!ok)) {
           if (et256 == 0) set_status(a.status, ST_TIMEOUT_EPI);
           *abort_flag = 1;
           break;
+        }
+        if (!settled) {
+          const int mine = bcast[0];
+          settle(mine);
+          if (mine != 3) {
+            rounds += staged ? 1 : 0;
+            continue;
+          }
         }
       }
 #pragma unroll 1

@@ -232,11 +232,11 @@ constexpr int kMaxAttnSplit = 16;       // key splits (CTAs of one cluster) of o
 // rows and at most kWideTok tokens, multiplied by a pair of CTAs.
 constexpr int kWideTok = 256;
 // A split tile's mask word: a bit per contributor that has stored its partial,
-// a bit per contributor that has given its share up, and above them the number
+// a bit per contributor whose given-up share nobody has claimed, and above them the number
 // of finished shares.
 constexpr int kWideContrib = 28, kWideReadShift = 2 * kWideContrib;
 // A contributor waits this long for the others of its tile before it gives its
-// share up to the last one to arrive (usually they arrive within 10 us): every
+// share up to one that arrives later (usually all arrive within 10 us): every
 // CTA of a launch ends in bounded time without the others, as it must where
 // launches of two streams share the SMs and neither is wholly on them.
 constexpr unsigned long long kShareWaitNs = 100000;
