@@ -7,10 +7,15 @@
 // 16 KB of weights.  Here a pair of CTAs (cta_group::2) shares a tile of 256
 // weight rows and up to 256 tokens: each CTA loads its own 128 weight rows
 // and half of the tokens, the tensor cores read the other half from the peer.
-// The hi and lo parts of a token go to the same accumulator column (two MMAs
-// per 16 columns of K, selected by the descriptors' atom stride), which
-// halves the accumulator: two 256-column buffers, so one tile's epilogue runs
-// under the next tile's MMAs.
+// Each 16 columns of K take two MMAs, one with the tokens' hi parts and one
+// with their lo parts (selected by the descriptors' atom stride).  The tensor
+// cores truncate at every accumulation, so hi and lo parts have accumulator
+// columns of their own wherever tensor memory holds two buffers of them (tiles
+// of at most 128 tokens), and in every tile of the QKV projection, whose keys
+// and values are rounded to bf16 (one buffer, the whole of tensor memory,
+// above 128 tokens).  The other projections' larger tiles sum both parts in
+// one column: two 256-column buffers, so one tile's epilogue runs under the
+// next tile's MMAs (sums a quarter as long changed the error of none of them).
 //
 // The tiles are shared out over the pairs whole, in equal parts or evenly by
 // K-steps, whichever is expected to end first (wide_split).  A tile split
@@ -67,9 +72,17 @@ __device__ __forceinline__ bool all_epi_any(bool v) {
   return r != 0;
 }
 
-// Epilogue values of one 16-token chunk straight from the accumulator
-__device__ __forceinline__ void load_acc(uint32_t taddr, float (&v)[kEpiTok]) {
+// Epilogue values of one 16-token chunk straight from the accumulator; lo: how
+// far behind the hi parts' columns the lo parts' are (0: in the same)
+__device__ __forceinline__ void load_acc(uint32_t taddr, int lo, float (&v)[kEpiTok]) {
   uint32_t r[16];
+  if (lo) {
+    uint32_t l[16];
+    tmem_ld16x2(taddr, taddr + lo, r, l);
+#pragma unroll
+    for (int j = 0; j < kEpiTok; ++j) v[j] = __uint_as_float(r[j]) + __uint_as_float(l[j]);
+    return;
+  }
   tmem_ld16(taddr, r);
 #pragma unroll
   for (int j = 0; j < kEpiTok; ++j) v[j] = __uint_as_float(r[j]);
@@ -94,6 +107,7 @@ static __device__ __noinline__ uint32_t give_share_up(unsigned long long* word, 
 template <int MODE>
 __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid_constant__ WideArgs w) {
   const GemmArgs& a = w.g;
+  constexpr bool kPieces = MODE == MODE_QKV;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + kWideRing);  // rank 0: both CTAs' stage has landed
@@ -141,6 +155,9 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   const int tok_tiles = live[0], n_tok = live[1];
+  // columns from the hi parts' accumulator to the lo parts' (0: one for both), and the buffers there are
+  const int lo = n_tok <= kWideTok / 2 ? kWideTok / 2 : MODE == MODE_QKV ? kWideTok : 0;
+  const int nacc = lo == kWideTok ? 1 : 2;
   const int kc = a.kc;
   // unit indices: 32 bits (the host checks that U times the pairs fits; 64-bit
   // divisions made up half of a short launch's tail)
@@ -153,8 +170,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
   // QKV: this pair's share [tb, te) of the tile of unit u is summed in pieces
   // of equal length, at most `chain` units each: the end of u's piece.
   auto piece_end = [&](int u, int tb, int te) {
-    if constexpr (MODE != MODE_QKV) return te;
-    const int chain = n_tok > 128 ? kWideChainPrompt : kWideChain;
+    if constexpr (!kPieces) return te;
+    const int chain = kc > kWideChain ? kWideChain : kWideChainShort;
     const int pieces = (te - tb + chain - 1) / chain, len = (te - tb + pieces - 1) / pieces;
     return min(tb + ((u - tb) / len + 1) * len, te);
   };
@@ -279,11 +296,11 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
       for (int u = u0; u < u1 && ok;) {
         const int tile0 = u / kc * kc;
         const int ub = u, ue = piece_end(u, max(tile0, u0), min(tile0 + kc, u1));
-        const int ab = seg_i & 1;
-        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&acce[ab], (uint32_t)((seg_i >> 1) & 1) ^ 1u, abort_flag));
+        const int ab = seg_i % nacc;
+        ok = __all_sync(0xffffffffu, mbar_wait_cluster(&acce[ab], (uint32_t)((seg_i / nacc) & 1) ^ 1u, abort_flag));
         if (!ok) break;
         tc_fence_after();
-        const uint32_t d = tmem + ab * kWideTok;
+        const uint32_t d = tmem + ab * kWideTok, dl = d + lo;
         for (; u < ue; ++u) {
           ok = __all_sync(0xffffffffu, mbar_wait(&full[s], fph, abort_flag));
           if (!ok) break;
@@ -294,8 +311,9 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
           if (elect_one()) {
 #pragma unroll
             for (int k = 0; k < kChunkK / 16; ++k) {
-              umma2_bf16(d, ad + 2 * k, bh + 2 * k, idesc, (u > ub || k > 0) ? 1u : 0u);
-              umma2_bf16(d, ad + 2 * k, bl + 2 * k, idesc, 1u);
+              const uint32_t more = (u > ub || k > 0) ? 1u : 0u;
+              umma2_bf16(d, ad + 2 * k, bh + 2 * k, idesc, more);
+              umma2_bf16(dl, ad + 2 * k, bl + 2 * k, idesc, lo ? more : 1u);
             }
             umma2_commit(&empty[s], 3);
             if (u + 1 == ue) umma2_commit(&accf[ab], 3);
@@ -404,7 +422,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         const int tb = max(t * kc, u0), te = min((t + 1) * kc, u1);
         const int ub = u, ue = piece_end(u, tb, te);
         u = ue;
-        ab = seg_i & 1;
+        ab = seg_i % nacc;
         wt0 = 2 * (t / tok_tiles) + (int)rank;
         tb0 = t % tok_tiles * n_tok;
         const int nch = chunks_of(wt0, tb0);
@@ -416,7 +434,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         const int slot = !whole && tb == u0 ? 0 : 1;
         float* mine = a.partials + ((size_t)(2 * c + rank) * 2 + slot) * kTileF;
         sum = ub > tb ? mine : nullptr;
-        ok = mbar_wait(&accf[ab], (uint32_t)((seg_i >> 1) & 1), abort_flag);
+        ok = mbar_wait(&accf[ab], (uint32_t)((seg_i / nacc) & 1), abort_flag);
         if (all_epi_any(!ok)) {
           if (et256 == 0) set_status(a.status, ST_TIMEOUT_EPI);
           *abort_flag = 1;
@@ -426,24 +444,37 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         tc_fence_after();
         tbase = tmem + ab * kWideTok + ((uint32_t)(q * 32) << 16);
         if (!whole || !last) {
-          // two chunks a turn: one accumulator read for both
+          // [chunk][j4][row] float4s: a warp's stores are 512 contiguous bytes
+          auto put = [&](float4* dst, float4 f) {
+            if (kPieces && sum) {
+              const float4 o = __ldcg(dst);  // this thread's own
+              f = make_float4(f.x + o.x, f.y + o.y, f.z + o.z, f.w + o.w);
+            }
+            *dst = f;
+          };
+          if (lo) {
 #pragma unroll 1
-          for (int ch = 2 * grp; ch < nch; ch += 4) {
-            uint32_t r[32];
-            tmem_ld32(tbase + ch * kEpiTok, r);
-            // [chunk][j4][row] float4s: a warp's stores are 512 contiguous bytes
-            float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kChF) + fr;
+            for (int ch = grp; ch < nch; ch += 2) {
+              float v[kEpiTok];
+              load_acc(tbase + ch * kEpiTok, lo, v);
+              float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kChF) + fr;
 #pragma unroll
-            for (int j4 = 0; j4 < 8; ++j4)
-              if (j4 < 4 || ch + 1 < nch) {
-                float4 f = make_float4(__uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
-                                       __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3]));
-                if (MODE == MODE_QKV && sum) {
-                  const float4 o = __ldcg(dst + j4 * kTileN);  // this thread's own
-                  f = make_float4(f.x + o.x, f.y + o.y, f.z + o.z, f.w + o.w);
-                }
-                dst[j4 * kTileN] = f;
-              }
+              for (int j4 = 0; j4 < 4; ++j4)
+                put(dst + j4 * kTileN, make_float4(v[4 * j4], v[4 * j4 + 1], v[4 * j4 + 2], v[4 * j4 + 3]));
+            }
+          } else {
+            // two chunks a turn: one accumulator read for both
+#pragma unroll 1
+            for (int ch = 2 * grp; ch < nch; ch += 4) {
+              uint32_t r[32];
+              tmem_ld32(tbase + ch * kEpiTok, r);
+              float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kChF) + fr;
+#pragma unroll
+              for (int j4 = 0; j4 < 8; ++j4)
+                if (j4 < 4 || ch + 1 < nch)
+                  put(dst + j4 * kTileN, make_float4(__uint_as_float(r[4 * j4]), __uint_as_float(r[4 * j4 + 1]),
+                                                     __uint_as_float(r[4 * j4 + 2]), __uint_as_float(r[4 * j4 + 3])));
+            }
           }
           tc_fence_before();
           // orders every thread's partial before the one release OR, and
@@ -592,8 +623,8 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
         tile_of(i, w_tile, tok0);
         float v[kEpiTok];
         if (from_acc) {
-          load_acc(tbase + i * kEpiTok, v);
-          if (MODE == MODE_QKV && sum) {
+          load_acc(tbase + i * kEpiTok, lo, v);
+          if (kPieces && sum) {
             const float4* p = reinterpret_cast<const float4*>(sum + (size_t)i * kChF) + fr;
 #pragma unroll
             for (int j4 = 0; j4 < 4; ++j4) {

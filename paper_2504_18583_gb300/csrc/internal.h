@@ -241,14 +241,17 @@ constexpr int kWideContrib = 28, kWideReadShift = 2 * kWideContrib;
 // launches of two streams share the SMs and neither is wholly on them.
 constexpr unsigned long long kShareWaitNs = 100000;
 // Units of the QKV projection that one accumulator sums before the epilogue
-// adds it up in fp32 registers: the tensor cores truncate at every
-// accumulation (hi and lo parts: eight a unit), and keys and values are
-// rounded to bf16 afterwards, so that small differences become whole
-// roundings.  Error against 64 bits, 4 layers of the 8B widths over a 512-row
-// prompt: 1.08e-3 with one accumulator per part and 64-token tiles, 1.11e-3
-// without a limit here, 1.02e-3 at 24 units, 0.99e-3 at 16 (the whole pass
-// 0.7% slower); a decode pass's 21 units stay in one piece.
-constexpr int kWideChain = 24, kWideChainPrompt = 16;
+// adds it up in fp32 registers (kWideChainShort where K has kWideChain or
+// fewer): the tensor cores truncate at every accumulation, and keys and values
+// are rounded to bf16 afterwards, so that small differences become whole
+// roundings.  Error against 64 bits: 6 layers of the 8B widths over a 512-row
+// prompt 1.37e-3 on 64-token tiles; here 1.27e-3 without a limit, 1.22e-3 at 32
+// units, 1.15e-3 at 16 (the pass 1.4% slower); 2 layers of the 70B widths
+// 1.53e-3, then 1.40e-3, 1.22e-3 and 1.14e-3; the draft pass of 8 sequences on
+// the 1B widths 1.007e-3, here 1.012e-3 in even shares of ten units, 0.994e-3
+// at 8.  Cutting the other projections' sums to 16 units changed no error and
+// made a 512-row pass 7% slower.
+constexpr int kWideChain = 32, kWideChainShort = 8;
 constexpr int kWideMaxRows = 2048;  // rows of one pass (64 sequences x 2 x 16)
 constexpr int kWideBoxL = 32, kWideBoxS = 16;
 struct WideArgs {

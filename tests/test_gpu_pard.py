@@ -522,3 +522,43 @@ def test_prompts_of_several_sequences_in_one_pass(lens):
         greedy_step(P, step)
     assert P.eng.last_status() == 0
     print("stats", P.stats)
+
+
+def test_wide_projection_rounds_values_as_often_right_as_the_narrow_one():
+    """The tensor cores truncate at every accumulation, and values are rounded
+    to bf16 after the projection: the share of a first layer's values that
+    differ from the correctly rounded 64-bit ones, from passes of up to 512
+    rows (CTA pairs) and from passes of 64 rows, on the 8B and 1B widths.
+    About 300 of 410k values differ; three standard deviations of a ratio of
+    two such counts are 3 sqrt(2 / 300) = 0.25."""
+    import torch
+    from paper_2504_18583_gb300 import pard
+    V, lens = 2056, (300, 100)
+    shapes = [s.replace(n_layers=1, vocab=V, mask_id=V - 1) for s in (S.TARGET_8B, S.DRAFT_1B)]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    weights, ref = [], []
+    prompts = [torch.randint(0, V - 1, (n,), generator=g, device="cuda").tolist() for n in lens]
+    for s in shapes:
+        w = {n: torch.empty(s.tensor_shape(n), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=g)
+             for n in S.GLOBAL_TENSORS + S.LAYER_TENSORS}
+        for n in ("attn_norm", "mlp_norm", "final_norm"):
+            w[n] += 1.0
+        h = [w["embed"][torch.tensor(p, device="cuda")].double() for p in prompts]
+        ref.append([((x / torch.sqrt((x * x).mean(-1, keepdim=True) + s.rms_eps) * w["attn_norm"].double())
+                     @ w["wv"].double().T).to(torch.bfloat16) for x in h])
+        weights.append({**{n: w[n] for n in S.GLOBAL_TENSORS}, "layers": [{n: w[n] for n in S.LAYER_TENSORS}]})
+    wrong = {}
+    for chunk in (512, 64):
+        for i, p in enumerate(prompts):  # passes of 300 and of 100 rows
+            eng = pard.PardEngine(shapes[0], weights[0], shapes[1], weights[1], max_batch=1, max_k=4, max_ctx=400,
+                                  n_pages=32, prefill_chunk=chunk)
+            eng.prefill([p], 8, 4)
+            for mi in (0, 1):
+                v = eng.read_kv(mi, 0, 0, list(range(len(p))), shapes[mi])[1].reshape(len(p), -1)
+                wrong[chunk, mi] = wrong.get((chunk, mi), 0) + int((v != ref[mi][i]).sum())
+            assert eng.last_status() == 0
+            eng.unpack_weights()
+            eng.close()
+    print(wrong)
+    for mi in (0, 1):
+        assert wrong[512, mi] <= 1.25 * wrong[64, mi], wrong
