@@ -446,9 +446,9 @@ __device__ __forceinline__ void store_pair8(__nv_bfloat16* x, int m, int col, in
   *reinterpret_cast<uint4*>(x + xpk(m, 0, col, x_rows)) = make_uint4(h[0], h[1], h[2], h[3]);
   *reinterpret_cast<uint4*>(x + xpk(m, 1, col, x_rows)) = make_uint4(l[0], l[1], l[2], l[3]);
 }
-// z / (1 + e^-z) with the hardware exponential and reciprocal: a few ulp of
-// fp32, against the 16 bits its hi/lo pair keeps of the product.
-__device__ __forceinline__ float silu(float z) { return __fdividef(z, 1.0f + __expf(-z)); }
+// z / (1 + e^-z): 1.6 ulp off at most over [-80, 80].  (With the hardware's
+// approximate exponential and quotient 31 ulp; passes were 1% to 2% faster.)
+__device__ __forceinline__ float silu(float z) { return z / (1.0f + expf(-z)); }
 
 // Warp reductions (fixed butterfly order, so results are deterministic).
 __device__ __forceinline__ float warp_sum(float v) {
