@@ -353,7 +353,11 @@ __device__ __forceinline__ void epi_chunk(const GemmArgs& a, float (&v)[kEpiTok]
       rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, 2));
       rmax = fmaxf(rmax, __shfl_xor_sync(0xffffffffu, rmax, 1));
       if (ri >= 0) {
-        const float least = rmax * 0.99f;
+        // Left out: entries whose score is below the best by more than the
+        // rough quotients' errors (1e-3 each) and an ulp of the score, which
+        // is rounded at the size of x / T (2^-23 of it): two scores that round
+        // to the same value are both in, so that the lower index wins.
+        const float least = rmax * (0.99f - 2.4e-7f * fabsf(T == 1.f ? mv : mv / T));
 #pragma unroll
         for (int k = 0; k < 16; ++k)
           if (in[k >> 2] && !(e[k] < least)) {  // NaN too

@@ -562,3 +562,50 @@ def test_wide_projection_rounds_values_as_often_right_as_the_narrow_one():
     print(wrong)
     for mi in (0, 1):
         assert wrong[512, mi] <= 1.25 * wrong[64, mi], wrong
+
+
+def flat_head_engine(batch, K):
+    """An engine whose draft gives every vocabulary entry the same logit: all
+    LM-head rows are one row."""
+    import torch
+    from paper_2504_18583_gb300 import pard
+    t, d = S.WORKLOADS["tiny"].target, S.WORKLOADS["tiny"].draft
+    g = torch.Generator(device="cuda").manual_seed(3)
+
+    def weights(s):
+        w = {n: torch.empty(s.tensor_shape(n), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=g)
+             for n in S.GLOBAL_TENSORS}
+        w["final_norm"] += 1.0
+        w["lm_head"][:] = w["lm_head"][0] * 8
+        w["layers"] = []
+        for _ in range(s.n_layers):
+            L = {n: torch.empty(s.tensor_shape(n), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=g)
+                 for n in S.LAYER_TENSORS}
+            L["attn_norm"] += 1.0
+            L["mlp_norm"] += 1.0
+            w["layers"].append(L)
+        return w
+
+    eng = pard.PardEngine(t, weights(t), d, weights(d), max_batch=batch, max_k=K, max_ctx=80, n_pages=5 * batch)
+    prompts = torch.randint(0, t.vocab - 1, (batch, 20), generator=torch.Generator().manual_seed(1)).tolist()
+    eng.prefill(prompts, 16, K)
+    return eng
+
+
+@pytest.mark.parametrize("batch,K,T", [(2, 4, 1e-7), (16, 6, 1e-7), (16, 6, 1e-6)])
+def test_sampled_draft_takes_the_lowest_index_of_equal_scores(batch, K, T):
+    """A Gumbel-max score is rounded at the size of logit / T: at a very low
+    temperature many entries share the best one, and the first of them is the
+    draw (16 and 96 rows: both GEMM kernels)."""
+    eng = flat_head_engine(batch, K)
+    out = eng.alloc_step_outputs(want_logits=True)
+    eng.draft(out, True, T, 77, 5)
+    d, z = out["draft"].cpu().numpy(), out["draft_logits"].cpu().numpy()
+    tied = 0
+    for b in range(batch):
+        for i in range(K):
+            sc = gumbel_scores(z[b, i], T, 77, STREAM_DRAFT, 5, b, i)
+            tied += int((sc == sc.max()).sum() > 1)
+            assert int(d[b, i]) == int(np.argmax(sc)), (b, i, int(d[b, i]), int(np.argmax(sc)), sc.max())
+    assert tied
+    assert eng.last_status() == 0
