@@ -298,6 +298,14 @@ int32_t pard_launch_count(pard_ctx* ctx);
 pard_status pard_attention_paths(pard_ctx* ctx, uint32_t* h_bits, void* stream);
 pard_status pard_set_attention_split_cap(pard_ctx* ctx, int32_t cap);
 
+/* Testing: how long a CTA pair that shares an output tile of a pass of more
+ * than 64 rows waits for the tile's other pairs before it gives its part of
+ * the finishing up to one that arrives later, in nanoseconds (0..1000000; -1
+ * restores the default 100000), from the next pass on.  Results do not
+ * depend on it, bit for bit: with 0 most parts change hands.  Returns
+ * PARD_ERR_ARG for a null context or another value. */
+pard_status pard_set_share_wait(pard_ctx* ctx, int32_t ns);
+
 /* Thread-local message for the last failing call ("" if none). */
 const char* pard_last_error(void);
 

@@ -268,6 +268,7 @@ struct pard_ctx {
   uint8_t* ws = nullptr;
   int sm = 0;
   int pairs = 0;          // CTA pairs of the wide GEMM the GPU holds at once
+  int share_wait_ns = kShareWaitNs;
   // activation buffers xd, xo, xf as tensors of 128-byte rows, in boxes of
   // 16, 32, .. 256 rows (the wide GEMM's half tiles)
   CUtensorMap xmap[3][kWideTok / 16];
@@ -349,6 +350,7 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
     w.x[0] = c->xmap[buf][a.n_tok / 16 - 1];
     w.x[1] = c->xmap[buf][kWideBoxL / 16 - 1];
     w.x[2] = c->xmap[buf][kWideBoxS / 16 - 1];
+    w.share_wait_ns = c->share_wait_ns;
     // a pass with fewer rows than its capacity splits its fewer tiles anew
     int pairs = 0;
     for (int tiles = 1; tiles <= (a.m_early ? a.tok_tiles : 1); ++tiles)
@@ -1264,6 +1266,13 @@ pard_status pard_set_attention_split_cap(pard_ctx* c, int32_t cap) {
   if (!c) return fail(PARD_ERR_ARG, "null context");
   if (cap < 0 || cap > kMaxAttnSplit) return fail(PARD_ERR_ARG, "attention split cap outside [0, 16]");
   c->attn_split_cap = cap == 0 ? kMaxAttnSplit : cap;
+  return PARD_OK;
+}
+
+pard_status pard_set_share_wait(pard_ctx* c, int32_t ns) {
+  if (!c) return fail(PARD_ERR_ARG, "null context");
+  if (ns < -1 || ns > 1000000) return fail(PARD_ERR_ARG, "share wait outside [-1, 1000000] ns");
+  c->share_wait_ns = ns < 0 ? kShareWaitNs : ns;
   return PARD_OK;
 }
 

@@ -568,7 +568,7 @@ __global__ void __launch_bounds__(kWideThreads, 1) gemm_wide_kernel(const __grid
             bool any = false;
             if (seen0 != all0) any |= fetch(sh0, all0, seen0, take0, 0, 0);
             if (seen1 != all1) any |= fetch(sh1, all1, seen1, take1, base1, 1);
-            if (!any && globaltimer() - t0 > kShareWaitNs) {
+            if (!any && globaltimer() - t0 > (unsigned)w.share_wait_ns) {
               // not in time: the round is done anew, without what is no longer this CTA's
               mine = 7;
               if (seen0 != all0) {

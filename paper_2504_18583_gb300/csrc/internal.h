@@ -239,7 +239,7 @@ constexpr int kWideContrib = 28, kWideReadShift = 2 * kWideContrib;
 // share up to one that arrives later (usually all arrive within 10 us): every
 // CTA of a launch ends in bounded time without the others, as it must where
 // launches of two streams share the SMs and neither is wholly on them.
-constexpr unsigned long long kShareWaitNs = 100000;
+constexpr int kShareWaitNs = 100000;
 // Units of the QKV projection that one accumulator sums before the epilogue
 // adds it up in fp32 registers (kWideChainShort where K has kWideChain or
 // fewer): the tensor cores truncate at every accumulation, and keys and values
@@ -257,6 +257,7 @@ constexpr int kWideBoxL = 32, kWideBoxS = 16;
 struct WideArgs {
   GemmArgs g;              // packed matrices: wmap holds the packed array as a tensor of 128-byte rows
   CUtensorMap x[3];        // the activation buffer as one, boxes of g.n_tok, kWideBoxL and kWideBoxS rows
+  int share_wait_ns;       // kShareWaitNs, or what a test asks for
 };
 // Token tiles of a pass of m rows, all of the same size (a multiple of 16).
 __host__ __device__ inline void wide_tiles(int m, int& tiles, int& n_tok) {

@@ -77,6 +77,8 @@ def lib() -> ctypes.CDLL:
         L.pard_attention_paths.restype = ctypes.c_int
         L.pard_set_attention_split_cap.argtypes = [vp, i32]
         L.pard_set_attention_split_cap.restype = ctypes.c_int
+        L.pard_set_share_wait.argtypes = [vp, i32]
+        L.pard_set_share_wait.restype = ctypes.c_int
         L.pard_unpack_weights.argtypes = [vp, vp]
         L.pard_unpack_weights.restype = ctypes.c_int
         L.pard_launch_count.argtypes = [vp]
@@ -319,3 +321,7 @@ class PardEngine:
     def set_attention_split_cap(self, cap: int) -> None:
         """At most `cap` key splits (CTAs of one cluster) per attention unit; 0: the default 16."""
         _check(lib().pard_set_attention_split_cap(self.ctx, int(cap)), "pard_set_attention_split_cap")
+
+    def set_share_wait(self, ns: int = -1) -> None:
+        """Testing: nanoseconds a CTA pair waits for the others of a shared output tile (-1: the default)."""
+        _check(lib().pard_set_share_wait(self.ctx, int(ns)), "pard_set_share_wait")

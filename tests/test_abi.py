@@ -83,3 +83,7 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, tmp_path):
     monkeypatch.setattr(pard, "_lib", None)
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         pard.lib()
+
+
+def test_share_wait_checks_its_arguments(lib):
+    assert lib.pard_set_share_wait(None, 0) == -1

@@ -609,3 +609,90 @@ def test_sampled_draft_takes_the_lowest_index_of_equal_scores(batch, K, T):
             assert int(d[b, i]) == int(np.argmax(sc)), (b, i, int(d[b, i]), int(np.argmax(sc)), sc.max())
     assert tied
     assert eng.last_status() == 0
+
+
+def random_engine(shapes, batch, K, prompt_len, seed=7, stream=None, prefill_chunk=512):
+    """An engine on seeded random weights (generated on the device), its prompts prefilled."""
+    import torch
+    from paper_2504_18583_gb300 import pard
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    weights = []
+    for s in shapes:
+        def mat(n):
+            t = torch.empty(s.tensor_shape(n), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=g)
+            return t + 1.0 if n.endswith("norm") else t
+        w = {n: mat(n) for n in S.GLOBAL_TENSORS}
+        w["layers"] = [{n: mat(n) for n in S.LAYER_TENSORS} for _ in range(s.n_layers)]
+        weights.append(w)
+    torch.cuda.synchronize()
+    pages = -(-(prompt_len + 16 + 2 * K) // 16)
+    eng = pard.PardEngine(shapes[0], weights[0], shapes[1], weights[1], max_batch=batch, max_k=K, stream=stream,
+                          max_ctx=prompt_len + 32 + 2 * K, n_pages=pages * batch, prefill_chunk=prefill_chunk)
+    p = torch.randint(0, shapes[0].vocab - 1, (batch, prompt_len), generator=torch.Generator().manual_seed(seed))
+    eng.prefill(p.tolist(), 16, K)
+    return eng
+
+
+def wide_pass(eng, out, cand):
+    eng.draft(out, True, 0.9, 5, 1)
+    eng.verify(out, cand, 1.0)
+    return [out[k].clone() for k in ("draft", "draft_logits", "logits")]
+
+
+WIDE_SHAPES = {
+    # model widths, sequences, K: rows and the split of the down projection's tiles
+    "odd_tiles": (dict(d_model=384, ffn=704, vocab=2056), 16, 7),
+    "26_pairs_a_tile": (dict(d_model=384, ffn=6656, vocab=2056), 16, 7),  # more partials than the ring has places
+    "two_token_tiles": (dict(d_model=512, ffn=2048, vocab=4096), 32, 9),
+    "8b_widths": (None, 16, 7),
+}
+
+
+@pytest.mark.parametrize("case", WIDE_SHAPES)
+def test_shared_tiles_do_not_depend_on_who_finishes_them(case):
+    """Passes of more than 64 rows in which CTA pairs give their parts of a
+    shared output tile up at once, after a microsecond, or not at all: the
+    same bits in every output, launch after launch."""
+    import torch
+    widths, batch, K = WIDE_SHAPES[case]
+    if widths:
+        t = S.WORKLOADS["tiny"].target.replace(n_layers=2, mask_id=widths["vocab"] - 1, **widths)
+        shapes = (t, t.replace(n_layers=1))
+    else:
+        shapes = [s.replace(n_layers=1, vocab=2056, mask_id=2055) for s in (S.TARGET_8B, S.DRAFT_1B)]
+    eng = random_engine(shapes, batch, K, 20)
+    out = eng.alloc_step_outputs(want_logits=True)
+    cand = torch.randint(0, shapes[0].vocab - 1, (batch, K), device="cuda", dtype=torch.int32)
+    want = wide_pass(eng, out, cand)
+    assert all(torch.isfinite(x.float()).all() for x in want)
+    for ns in (0, 0, 0, 700, 0, 1000, -1, 0, -1):
+        eng.set_share_wait(ns)
+        for got, w in zip(wide_pass(eng, out, cand), want):
+            assert torch.equal(got, w), ns
+    assert eng.last_status() == 0
+
+
+def test_two_engines_on_two_streams():
+    """Two engines whose passes of more than 64 rows run at the same time on
+    streams of their own: each gives the bits that it gives alone."""
+    import torch
+    shapes = [s.replace(n_layers=2, vocab=4104, mask_id=4103) for s in (S.TARGET_8B, S.DRAFT_1B)]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    cand = torch.randint(0, 4103, (16, 6), device="cuda", dtype=torch.int32)
+    torch.cuda.synchronize()
+    engines = [random_engine(shapes, 16, 6, 40, seed=k, stream=s) for k, s in enumerate(streams)]
+    outs, alone = [], []
+    for e, s in zip(engines, streams):
+        with torch.cuda.stream(s):
+            outs.append(e.alloc_step_outputs(want_logits=True))
+            alone.append(wide_pass(e, outs[-1], cand))
+        torch.cuda.synchronize()
+    for _ in range(6):
+        got = []
+        for e, s, o in zip(engines, streams, outs):
+            with torch.cuda.stream(s):
+                got.append(wide_pass(e, o, cand))
+        torch.cuda.synchronize()
+        for a, b in zip(alone, got):
+            assert all(torch.equal(x, y) for x, y in zip(a, b))
+    assert [e.last_status() for e in engines] == [0, 0]
