@@ -696,3 +696,27 @@ def test_two_engines_on_two_streams():
         for a, b in zip(alone, got):
             assert all(torch.equal(x, y) for x, y in zip(a, b))
     assert [e.last_status() for e in engines] == [0, 0]
+
+
+@pytest.mark.parametrize("T", [0.05, 0.7, 1.0, 1.3])
+@pytest.mark.parametrize("batch,K", [(2, 4), (8, 4), (16, 6)], ids=["16_rows", "64_rows", "192_rows"])
+def test_lm_head_draw_follows_its_own_logits(batch, K, T):
+    """The draw that the draft pass makes in the LM head (a rough ranking,
+    then exact scores of the few best): the token of the highest Gumbel score
+    of the logits the pass returns, except where the lead is within the
+    roundings of the two sides' noise and of the sum."""
+    t = S.WORKLOADS["tiny"].target.replace(n_layers=1, vocab=4104, mask_id=4103)
+    eng = random_engine((t, t), batch, K, 20, seed=int(100 * T))
+    out = eng.alloc_step_outputs(want_logits=True)
+    near = 0
+    for step in (1, 2):
+        eng.draft(out, True, T, 91, step)
+        d, z = out["draft"].cpu().numpy(), out["draft_logits"].cpu().numpy()
+        for b in range(batch):
+            for i in range(K):
+                sc = gumbel_scores(z[b, i], T, 91, STREAM_DRAFT, step, b, i)
+                if int(d[b, i]) != int(np.argmax(sc)):
+                    assert sc[d[b, i]] >= sc.max() - GUMBEL_EPS - 2 * np.spacing(np.abs(sc).max()), (step, b, i)
+                    near += 1
+    assert near <= 2
+    assert eng.last_status() == 0

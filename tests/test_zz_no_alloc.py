@@ -95,3 +95,43 @@ def test_noalloc_tile_edges_masked_rows_and_unaligned_logits(vocab):
                              else OP.accept_greedy(d[b], y[b]))
             assert int(acc[b]) == a_o, (sample, b)
             assert em[b].tolist()[:a_o + 1] == [int(t) for t in em_o], (sample, b)
+
+
+@pytest.mark.parametrize("T", [1e-3, 0.05, 0.7, 1.3])
+def test_noalloc_sampling_at_other_temperatures(T):
+    """Temperatures other than 1, down to scores of several thousand (where
+    the draw's sum is rounded to 1e-3 and several entries can share the best
+    score): accept lengths and tokens of the oracle's rule, the bonus token
+    except where its lead is within the two sides' roundings."""
+    import torch
+    from _parity import GUMBEL_EPS, gumbel_scores
+    from oracle.philox import STREAM_BONUS
+    from paper_2504_18583_gb300 import _build, pard
+    _build.build()
+    B, K, vocab = 16, 3, 4104
+    rng = np.random.default_rng(int(T * 1000))
+    y = (rng.standard_normal((B, K + 1, vocab)) * 2.0).astype(np.float32)
+    y[: B // 2] = np.round(y[: B // 2])  # many equal logits
+    z = y[:, :K] + (T * rng.standard_normal((B, K, vocab))).astype(np.float32)
+    z[: B // 4] = y[: B // 4, :K]  # p = q: every candidate is accepted, the bonus comes from the last row
+    d = np.array([OP.draft_tokens(z[b], True, T, 8, 4, b) for b in range(B)], dtype=np.int32)
+    yt, zt, dt = (torch.as_tensor(a, device="cuda") for a in (y, z, d))
+    acc = torch.empty(B, dtype=torch.int32, device="cuda")
+    em = torch.empty((B, K + 1), dtype=torch.int32, device="cuda")
+    code = pard.lib().pard_accept_noalloc(yt.data_ptr(), zt.data_ptr(), dt.data_ptr(), B, K, vocab, 1, T, 21, 4,
+                                          acc.data_ptr(), em.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    assert code == 0, pard.pard_last_error()
+    exact = 0
+    for b in range(B):
+        with np.errstate(divide="ignore", invalid="ignore"):
+            a_o, em_o = OP.accept_sampling(d[b], z[b], y[b], T, 21, 4, b)
+        assert int(acc[b]) == a_o, b
+        got = em[b].tolist()[:a_o + 1]
+        assert got[:a_o] == [int(x) for x in em_o[:a_o]], b
+        if got[a_o] == int(em_o[a_o]):
+            exact += 1
+        elif a_o == K:
+            sc = gumbel_scores(y[b, K], T, 21, STREAM_BONUS, 4, b, 0)
+            assert sc[got[a_o]] >= sc.max() - GUMBEL_EPS - 2 * np.spacing(np.abs(sc).max()), b
+    assert exact >= B - 1
+    assert (acc.cpu().numpy()[: B // 4] == K).all()
