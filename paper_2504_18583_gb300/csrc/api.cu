@@ -319,9 +319,9 @@ GemmArgs gemm_base(pard_ctx* c, int rows_cap, int tt) {
   std::memset(&a, 0, sizeof(a));
   if (tt == kWideTok) {
     wide_tiles(rows_cap, a.tok_tiles, a.n_tok);
-  } else {
-    a.tok_tiles = (rows_cap + tt - 1) / tt;
-    a.n_tok = a.tok_tiles == 1 ? round_up(rows_cap, 8) : 0;
+  } else {  // rows_cap <= tt
+    a.tok_tiles = 1;
+    a.n_tok = round_up(rows_cap, 8);
   }
   a.m_cap = c->D.MC;
   a.m_dev = c->rp.m_dev;
@@ -359,13 +359,12 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
     c->launches++;
     return;
   }
-  const long U = (long)a.w_tiles * a.tok_tiles * a.kc;
+  const long T = a.w_tiles, U = T * a.kc;
   // At least 8 units (128 KB of weights) a CTA: with fewer, the split-K
   // finish of a tile gathers partials from too many CTAs; and at least
   // kc / 62 units, so that no tile has more than 63 contributors (the
   // finisher tracks their arrivals in one 64-bit mask).  But a tile is never
   // shared for that (tiny configuration's verify pass: 104 -> 82 us).
-  const long T = (long)a.w_tiles * a.tok_tiles;
   const long min_units = std::max<long>(8, (a.kc + 61) / 62);
   const long most = std::min<long>(c->sm, std::max<long>(U / min_units, T));
   long grid = most;
@@ -378,11 +377,12 @@ void run_gemm(pard_ctx* c, GemmArgs& a, int tt, cudaStream_t s) {
     // One or two whole tiles a CTA and no exchange at all: two CTAs of the
     // 16-token tile fit on an SM, and as all wait for HBM they end together
     // although some SMs hold two (8B verify pass 2890 -> 2827 us, 70B widths
-    // 1472 -> 1454).
+    // 1472 -> 1454).  More tiles than two an SM in an odd number do not pair
+    // up and keep the even split.
     if (T <= 2 * c->sm) grid = T;
     else if (T % 2 == 0) grid = T / 2;
   }
-  if ((long)a.w_tiles * a.tok_tiles > kMaxGemmTiles || (U + 1) * (grid + 1) > INT32_MAX) throw cudaErrorInvalidValue;
+  if (T > kMaxGemmTiles || (U + 1) * (grid + 1) > INT32_MAX) throw cudaErrorInvalidValue;
   launch_gemm(a, tt, (int)grid, s, true);
   c->launches++;
 }
@@ -486,7 +486,7 @@ LayerPlan layer_plan(pard_ctx* c, int mi, int l, int rows_cap, int tt, int batch
     a.page_table = pt_attn; a.pt_ld = c->D.pt_ld;
     a.row_pos = c->rp.row_pos; a.seq_row0 = c->rp.seq_row0; a.rows_per_seq = fixed_rows; a.m_dev = c->rp.m_dev;
     a.batch = batch; a.hq = cf.n_q_heads; a.hkv = cf.n_kv_heads; a.hd = cf.head_dim;
-    a.page_size = c->lim.page_size; a.n_pages = c->lim.n_pages;
+    a.n_pages = c->lim.n_pages;
     a.row_blocks = geo.row_blocks; a.n_split = geo.n_split;
     a.nbuf = geo.nbuf;
     a.prompt = geo.prompt;

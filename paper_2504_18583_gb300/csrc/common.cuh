@@ -37,31 +37,12 @@ __device__ __forceinline__ unsigned long long globaltimer() {
   return t;
 }
 
-// atomic add at GPU scope with release and acquire semantics; returns the old value
-__device__ __forceinline__ int atom_add_acq_rel(int* p, int v) {
-  int old;
-  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-  return old;
-}
-
-__device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ int ld_acquire_s32(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
+// atomics at GPU scope with release and acquire semantics; they return the old value
 __device__ __forceinline__ unsigned long long atom_or64(unsigned long long* p, unsigned long long v) {
   unsigned long long old;
   asm volatile("atom.acq_rel.gpu.global.or.b64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
@@ -75,8 +56,6 @@ __device__ __forceinline__ unsigned long long atom_and64(unsigned long long* p, 
 __device__ __forceinline__ void red_release_or64(unsigned long long* p, unsigned long long v) {
   asm volatile("red.release.gpu.global.or.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-// with a preceding relaxed read that saw a released value: acquire
-__device__ __forceinline__ void fence_acq_rel_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 // orders this thread's generic-proxy global accesses with its async-proxy (bulk copy) ones
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
@@ -221,13 +200,6 @@ __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap* m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
 }
 // 2-D tiled load of one box into shared memory; completion is counted on bar.
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1), "r"(smem_u32(bar))
-      : "memory");
-}
 __device__ __forceinline__ void tma_load_2d_hint(void* dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1,
                                                  uint64_t policy) {
   asm volatile(
@@ -402,13 +374,8 @@ __host__ __device__ __forceinline__ size_t xpk(int m, int lo, int k, int two_row
 // Weights: a matrix [N][K] packed in blocks of R rows: [N/R][K/64][R][64], the
 // same 128-byte swizzle inside each R x 64 block (R = 128, or 64 for the
 // gate/up halves).
-__host__ __device__ __forceinline__ size_t wpk(int n, int k, int R, int K) {
-  const int b = n / R, r = n % R;
-  return (((size_t)b * (K >> 6) + (k >> 6)) * R + r) * 64 + (size_t)((((k & 63) >> 3) ^ (r & 7)) << 3) + (k & 7);
-}
 
 // ---- numerics --------------------------------------------------------------
-__device__ __forceinline__ float bf16_bits_to_f32(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 // split x into hi + lo with both parts bf16 (hi = RNE(x), lo = RNE(x - hi))
 __device__ __forceinline__ void split_bf16(float x, __nv_bfloat16& hi, __nv_bfloat16& lo) {
   hi = __float2bfloat16_rn(x);

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = gridDim.x;
   const int c = blockIdx.x;
-  const int tok_tiles = a.tok_tiles, U = a.w_tiles * tok_tiles * a.kc;
+  const int U = a.w_tiles * a.kc;  // one token tile
   const int u0 = range_start(c, U, G), u1 = range_start(c + 1, U, G);  // this CTA's units
 
   if (threadIdx.x == 0) {
@@ -78,11 +78,9 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   uint32_t armed = 0, armed_odd = 0;  // producer: slots armed at least once, and those armed an odd number of times
-  // ring slots this launch uses, and how many are filled before the PDL wait
-  const int R = (a.stages > 0 && a.stages < C::kStages) ? a.stages : C::kStages;
-  const int P = (a.pre_stages > 0 && a.pre_stages < R) ? a.pre_stages : R;
+  constexpr int R = C::kStages;
   // token rows a tile's MMA covers: hi/lo pairs are the B rows, so N = 2 n_tok
-  const int n_tok = (tok_tiles == 1 && a.n_tok > 0 && a.n_tok < TT && a.n_tok % 8 == 0) ? a.n_tok : TT;
+  const int n_tok = min(a.n_tok, TT);
   const uint32_t b_bytes = (uint32_t)n_tok * 2 * 128;
   const uint32_t stage_bytes = (uint32_t)C::kABytes + b_bytes;
 
@@ -93,12 +91,12 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
     {
       const uint64_t pol = policy_evict_first();
       const int n = u1 - u0;
-      const int npre = n < P ? n : P;
+      const int npre = n < R ? n : R;
       // Unit cursor advanced incrementally: the producer issues one stage per
       // wake-up with no divisions on the path between the 'empty' signal and
       // the copies.
       int kk = u0 % a.kc;
-      int w_tile = u0 / a.kc / tok_tiles, tok_tile = u0 / a.kc % tok_tiles;
+      int w_tile = u0 / a.kc;
       const __nv_bfloat16* wsrc0 = nullptr;  // packed block base of the current weight tile (A)
       const __nv_bfloat16* wsrc1 = nullptr;  // second half (gate/up pairs)
       const CUtensorMap* wmap0 = nullptr;
@@ -121,7 +119,6 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
         }
       };
       set_tile();
-      const size_t x_tile_off = (size_t)2 * TT * 64;      // elements between token tiles of one block
       const size_t x_blk = (size_t)a.x_rows * 64;         // elements between 64-column blocks
       auto issue_a = [&](int s) {
         uint8_t* dst = sA + s * C::kABytes;
@@ -139,13 +136,13 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
           tma_load_2d_hint(dst, wmap0, &full[s], kk * kChunkK, wrow, pol);
         }
       };
-      auto issue_b = [&](int s, int kk_, int tok_) {
-        bulk_load(sB + s * C::kBBytes, a.x + (size_t)kk_ * x_blk + (size_t)tok_ * x_tile_off, b_bytes, &full[s]);
+      auto issue_b = [&](int s, int kk_) {
+        bulk_load(sB + s * C::kBBytes, a.x + (size_t)kk_ * x_blk, b_bytes, &full[s]);
       };
       auto advance = [&]() {
         if (++kk == a.kc) {
           kk = 0;
-          if (++tok_tile == tok_tiles) { tok_tile = 0; ++w_tile; }
+          ++w_tile;
           set_tile();
         }
       };
@@ -154,7 +151,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
         armed |= 1u << s;
         armed_odd ^= 1u << s;
       };
-      const int kk0 = kk, tok0 = tok_tile;
+      const int kk0 = kk;
       for (int i = 0; i < npre; ++i) {
         arm(i);
         if (elect_one()) {
@@ -165,10 +162,10 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
         advance();
       }
       pdl_wait();
-      for (int i = 0, k2 = kk0, t2 = tok0; i < npre; ++i) {
-        if (elect_one()) issue_b(i, k2, t2);
+      for (int i = 0, k2 = kk0; i < npre; ++i) {
+        if (elect_one()) issue_b(i, k2);
         __syncwarp();
-        if (++k2 == a.kc) { k2 = 0; if (++t2 == tok_tiles) t2 = 0; }
+        if (++k2 == a.kc) k2 = 0;
       }
       int s = npre % R;
       uint32_t ph = (uint32_t)((npre / R) & 1) ^ 1u;
@@ -182,7 +179,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
         if (elect_one()) {
           mbar_arrive_expect_tx(&full[s], stage_bytes);
           issue_a(s);
-          issue_b(s, kk, tok_tile);
+          issue_b(s, kk);
         }
         __syncwarp();
         advance();
@@ -242,22 +239,16 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
       M = a.m_cap;
     }
     int seg_i = 0;
-    int rs_tok = -1;  // token tile whose RMS row scale S.rs holds
+    if (MODE != MODE_RESID && u0 < u1) epi_row_scale<TT>(a, et, M, S);
     for (int u = u0; u < u1;) {
       const int t = u / a.kc;
       const int ub = u, ue = (t + 1) * a.kc < u1 ? (t + 1) * a.kc : u1;
       u = ue;
       const int ab = seg_i % C::kNumAcc;
-      const int w_tile = t / tok_tiles, tok_tile = t % tok_tiles;
-      const int tok_base = tok_tile * TT;
-      if (MODE != MODE_RESID && tok_base != rs_tok) {
-        epi_row_scale<TT>(a, tok_base, et, M, S);
-        rs_tok = tok_base;
-      }
       // result-independent loads of a segment this CTA finishes (it starts
       // the tile), issued while the MMAs run
       EpiPre pre0 = {};
-      if (ub == t * a.kc) pre0 = epi_pre<MODE>(a, w_tile, tok_base, et, M);
+      if (ub == t * a.kc) pre0 = epi_pre<MODE>(a, t, 0, et, M);
       if (!mbar_wait(&accf[ab], (uint32_t)((seg_i / C::kNumAcc) & 1), abort_flag)) {
         if (et == 0) set_status(a.status, ST_TIMEOUT_EPI);
         *abort_flag = 1;
@@ -266,7 +257,7 @@ __global__ void __launch_bounds__(192, TT <= 16 ? 2 : 1) gemm_kernel(const __gri
       tc_fence_after();
       epi_bar();
       const uint32_t tbase = tmem + ab * C::kAccCols + ((uint32_t)(q * 32) << 16);
-      if (!epi_segment_owned<TT, MODE>(a, t, ub, ue, u0, U, G, c, tbase, w_tile, tok_base, fr, et, M, S, pre0,
+      if (!epi_segment_owned<TT, MODE>(a, t, ub, ue, u0, U, G, c, tbase, fr, et, M, S, pre0,
                                  reinterpret_cast<float*>(sA), (uint32_t)(C::kStages * C::kStageBytes), fx,
                                  fx_armed, abort_flag, bcast))
         break;

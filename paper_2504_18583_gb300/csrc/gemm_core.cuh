@@ -421,26 +421,26 @@ __device__ __forceinline__ int chunk_groups(int M, int tok0) { return min(4, max
 // fewer) and are cleared by the finisher.
 template <int TT, int MODE>
 __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int u0, int U, int G, int c,
-                                  uint32_t tbase, int w_tile, int tok_base, int fr, int et, int M, const EpiSmem& S,
+                                  uint32_t tbase, int fr, int et, int M, const EpiSmem& S,
                                   const EpiPre& pre0, float* ring, uint32_t ring_bytes, uint64_t* fx,
                                   volatile int* fx_armed, volatile int* abort_flag, int* bcast) {
   using C = GemmCfg<TT>;
   constexpr int kTileF = kTileN * TT;  // floats of one partial tile
   // 16-token chunks holding at least one of the pass's M rows; the others are
   // neither finished nor exchanged (their rows are not outputs)
-  const int nch = max(0, min(C::kChunks, (M - tok_base + kEpiTok - 1) / kEpiTok));
+  const int nch = max(0, min(C::kChunks, (M + kEpiTok - 1) / kEpiTok));
   const int kChF = kTileN * kEpiTok;   // floats of one chunk of a partial tile
   if (ub == t * a.kc && ue == (t + 1) * a.kc) {
     EpiPre pre = pre0;  // one chunk's loads live at a time
 #pragma unroll 1
     for (int ch = 0; ch < nch; ++ch) {
-      if (ch > 0) pre = epi_pre<MODE>(a, w_tile, tok_base + ch * kEpiTok, et, M);
+      if (ch > 0) pre = epi_pre<MODE>(a, t, ch * kEpiTok, et, M);
       uint32_t r[32];
       tmem_ld32(tbase + ch * 32, r);
       float v[kEpiTok];
 #pragma unroll
       for (int j = 0; j < kEpiTok; ++j) v[j] = hilo(r, j);
-      epi_chunk<MODE>(a, v, w_tile, tok_base + ch * kEpiTok, ch * kEpiTok, fr, et, M, S, pre);
+      epi_chunk<MODE>(a, v, t, ch * kEpiTok, ch * kEpiTok, fr, et, M, S, pre);
     }
     return true;
   }
@@ -453,7 +453,7 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
     for (int ch = 0; ch < nch; ++ch) {
       uint32_t r[32];
       tmem_ld32(tbase + ch * 32, r);
-      const int ng = chunk_groups(M, tok_base + ch * kEpiTok);
+      const int ng = chunk_groups(M, ch * kEpiTok);
       // [chunk][j4][row] float4s: a warp's accesses are 512 contiguous bytes
       float4* dst = reinterpret_cast<float4*>(mine + (size_t)ch * kTileN * kEpiTok) + fr;
 #pragma unroll
@@ -473,7 +473,7 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
     // ring_bytes / 8 KB contributors) or direct loads
     const int n_other = cl - cf;
     // bytes copied of one contributor: the 4-token groups of its chunk with output rows
-    const uint32_t part_bytes = nch > 0 ? (uint32_t)chunk_groups(M, tok_base) * kTileN * 16 : 0u;
+    const uint32_t part_bytes = nch > 0 ? (uint32_t)chunk_groups(M, 0) * kTileN * 16 : 0u;
     const bool staged = nch > 0 && (uint32_t)n_other * kChF * 4 <= ring_bytes;
     if (et == 0) {
       const unsigned long long all = contrib_bits(n_other);
@@ -523,7 +523,7 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
     EpiPre pre = pre0;
   #pragma unroll 1
     for (int ch = 0; ch < nch; ++ch) {
-      if (ch > 0) pre = epi_pre<MODE>(a, w_tile, tok_base + ch * kEpiTok, et, M);
+      if (ch > 0) pre = epi_pre<MODE>(a, t, ch * kEpiTok, et, M);
       uint32_t r[32];
       tmem_ld32(tbase + ch * 32, r);
       float v[kEpiTok];
@@ -550,7 +550,7 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
           v[4 * j4 + 3] += pv[j4].w;
         }
       }
-      epi_chunk<MODE>(a, v, w_tile, tok_base + ch * kEpiTok, ch * kEpiTok, fr, et, M, S, pre);
+      epi_chunk<MODE>(a, v, t, ch * kEpiTok, ch * kEpiTok, fr, et, M, S, pre);
     }
   } else {
     const int n_other = cl - cf;
@@ -599,7 +599,7 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
       }
   #pragma unroll 1
       for (int ch = r0; ch < r1; ++ch) {
-        if (ch > 0) pre = epi_pre<MODE>(a, w_tile, tok_base + ch * kEpiTok, et, M);
+        if (ch > 0) pre = epi_pre<MODE>(a, t, ch * kEpiTok, et, M);
         uint32_t r[32];
         tmem_ld32(tbase + ch * 32, r);
         float v[kEpiTok];
@@ -626,7 +626,7 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
             v[4 * j4 + 3] += pv[j4].w;
           }
         }
-        epi_chunk<MODE>(a, v, w_tile, tok_base + ch * kEpiTok, ch * kEpiTok, fr, et, M, S, pre);
+        epi_chunk<MODE>(a, v, t, ch * kEpiTok, ch * kEpiTok, fr, et, M, S, pre);
       }
       if (staged && r1 < nch) epi_bar();  // the ring is read out before the next round's copies
     }
@@ -635,15 +635,15 @@ __device__ bool epi_segment_owned(const GemmArgs& a, int t, int ub, int ue, int 
   return true;
 }
 
-// RMS row scale for the token tile starting at tok_base: all partial sums of
-// squares in one round of loads, then a fixed-order sum per row.
+// RMS row scales of the pass's rows: all partial sums of squares in one round
+// of loads, then a fixed-order sum per row.
 template <int TT>
-__device__ void epi_row_scale(const GemmArgs& a, int tok_base, int et, int M, const EpiSmem& S) {
+__device__ void epi_row_scale(const GemmArgs& a, int et, int M, const EpiSmem& S) {
   for (int c0 = 0; c0 < TT; c0 += kEpiTok) {
     const int nld = a.ssq_tiles * kEpiTok;
     for (int i = et; i < nld; i += 128) {
       const int tile = i / kEpiTok, j = i % kEpiTok;
-      const int m = tok_base + c0 + j;
+      const int m = c0 + j;
       S.xch[i] = m < M ? __ldcg(a.ssq_in + (size_t)tile * a.m_cap + m) : 0.f;
     }
     epi_bar();

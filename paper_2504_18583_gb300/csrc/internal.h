@@ -40,9 +40,9 @@ struct GemmArgs {
   int seg_tile0[kMaxSeg + 1]; // prefix sums of tiles per segment
   int seg_rows[kMaxSeg];      // rows of each segment
   int pair;
-  int w_tiles, tok_tiles, kc;
-  int n_tok;                  // token rows a tile's MMA covers (multiple of 8, <= the tile; 0: the whole tile):
-                              // a single-tile pass of fewer rows loads and multiplies only those
+  int w_tiles, tok_tiles, kc; // tok_tiles: 1 in the narrow GEMM
+  int n_tok;                  // token rows a tile's MMA covers (multiple of 8, <= the tile): a pass of fewer rows
+                              // loads and multiplies only those
   int m_early;                // wide GEMM: m_dev was written two or more launches back, so it is read before the
                               // PDL wait, and the token tiles are laid out for the rows there are
   int mode;
@@ -52,8 +52,6 @@ struct GemmArgs {
   int* counters;              // split-K arrival masks: 64-bit word per output tile, zero between launches
   uint32_t* status;
   int max_pairs;              // wide GEMM: pairs the GPU holds at once
-  int stages;                 // ring slots used (0: all the kernel has)
-  int pre_stages;             // slots filled before waiting on the previous kernel (0: stages)
   // RMS row scale applied after the reduction (null: none)
   const float* ssq_in;
   int ssq_tiles;
@@ -99,7 +97,7 @@ struct AttnArgs {
   int rows_per_seq;           // > 0: every sequence has this many rows (row0 = b x it), seq_row0 unread
   const int* m_dev;
   int batch;
-  int hq, hkv, hd, page_size, n_pages;
+  int hq, hkv, hd, n_pages;   // pages of kAttnPage tokens
   int row_blocks;             // row blocks per sequence (grid.y / ...)
   int n_split;                // key splits
   int prompt;                 // a prompt pass: units are launched longest first
