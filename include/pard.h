@@ -129,7 +129,12 @@ pard_status pard_load_weights(pard_ctx** out, const pard_model_cfg* target, cons
  * decoding with the target alone (Eq. 2): each pard_verify runs one row per
  * sequence and pard_accept_commit emits its argmax (or a draw from it), and
  * pard_draft returns PARD_ERR_STATE; it is the baseline the paper's speedups
- * are measured against.  Synchronises `stream`. */
+ * are measured against.
+ * The prompts are one run of rows, taken prefill_chunk at a time whichever
+ * prompts they belong to: like a decode pass's, the results of a sequence are
+ * the same bits for the same batch, and may differ in their last bits (within
+ * the precision of the pass) with the other prompts of the batch.
+ * Synchronises `stream`. */
 pard_status pard_prefill(pard_ctx* ctx, const int32_t* d_tokens, const int32_t* h_lens, int32_t batch,
                          int32_t n_new, int32_t K, int32_t sample, float temperature, uint64_t seed,
                          int32_t* d_first_token, void* stream);
@@ -255,8 +260,10 @@ pard_status pard_unpack_weights(pard_ctx* ctx, void* stream);
  * counterpart: this is an interface for callers that cannot provide device
  * memory of their own -- runtimes without a device allocator, or engines that
  * plan all device memory ahead and forbid allocation on their serving path.
- * Inputs and outputs are as for pard_set_logits + pard_accept_commit (the
- * same kernels, same results): d_target_logits [batch][K+1][vocab],
+ * Inputs and outputs are as for pard_set_logits + pard_accept_commit, by the
+ * same rule and the same draws.  The normalisers of the rows are summed in
+ * tiles of another size, so where a sampled decision or draw hangs on the last
+ * bits of one the two may differ: d_target_logits [batch][K+1][vocab],
  * d_draft_logits [batch][K][vocab] (needed only when sample != 0), d_draft
  * [batch][K]; outputs d_accept_len [batch] and d_emitted [batch][K+1] (-1
  * after the emitted tokens).  A candidate outside [0, vocab) is never read

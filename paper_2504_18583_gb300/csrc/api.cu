@@ -255,7 +255,12 @@ CUtensorMap make_map(const void* base, size_t rows, int cols, int box_rows, bool
 }
 
 // Token tile of a pass of up to `rows` rows: 16, 64, or (more) the wide
-// kernel's, kWideTok.
+// kernel's, kWideTok.  The host knows a draft pass's capacity, 2 K rows a
+// sequence, not its rows (K to 2 K), so one of 64 rows or fewer may take the
+// wide kernel.  1B draft, K = 8, at 40 / 56 / 64 rows of a capacity of 80 /
+// 112 / 128: 1161 / 1175 / 1179 us; 64-token tiles that skipped the empty one
+// took 1452 / 1628 / 1648.  Within a capacity of 64 rows it is the slower one
+// at 18 rows (1B draft 834 -> 1098 us) and level at 63.
 int pick_tt(int rows) { return rows <= 16 ? 16 : (rows <= 64 ? 64 : kWideTok); }
 
 }  // namespace

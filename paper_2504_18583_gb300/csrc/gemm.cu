@@ -1,8 +1,9 @@
-// Weight-streaming GEMM for the decode step: Y[m][n] = sum_k X[m][k] W[n][k]
+// Weight-streaming GEMM of passes of up to 64 rows: Y[m][n] = sum_k X[m][k] W[n][k]
 // with W bf16 [N][K] streamed from HBM exactly once per launch and X a few
 // activation rows (M = K+1 verify rows, up to 2K draft rows per sequence).
 //
-// GB300 design (one CTA per SM, persistent, stream-K):
+// GB300 design (one launch fills the GPU once; one CTA per SM, two where tiles
+// of 16 tokens are shared out whole):
 //  * operand swap: the weight tile is the UMMA A operand (M = 128 weight
 //    rows), the activations the B operand (N = 2 x token tile), so a skinny
 //    M=9 product still issues full 128-row tensor-core tiles;
@@ -14,11 +15,12 @@
 //    with TMA (128-byte swizzle) through a multi-stage mbarrier ring, warp 1
 //    issues tcgen05.mma into a TMEM accumulator, warps 2-5 drain TMEM;
 //  * the flattened (tile, K-chunk) index space is split evenly over the
-//    CTAs; a tile shared by several CTAs is finished by the first of them,
-//    for which it is the last segment: the others store their partials and
-//    signal with one release increment each, the finisher pulls all partials
-//    into its idle stage ring with bulk copies and sums them in CTA order
-//    (deterministic);
+//    CTAs, in whole tiles or with every tile in the same number of parts
+//    (run_gemm chooses the number of CTAs so); a tile shared by several CTAs
+//    is finished by the first of them, for which it is the last segment: the
+//    others store their partials and set their bit of the tile's mask with one
+//    release OR each, the finisher pulls all partials into its idle stage ring
+//    with bulk copies and sums them in CTA order (deterministic);
 //  * epilogues are fused: RMS row scaling, RoPE + paged KV write (QKV),
 //    residual add + next norm's gain and sum of squares (O / down),
 //    SiLU(gate) * up (gate/up pairs), logits + per-tile max / argmax /

@@ -37,7 +37,7 @@
 // QKV 36 -> 24, O 30 -> 23, gate/up 62 -> 52 (34 at the HBM rate), down 52 -> 36,
 // LM head 236 -> 183; 512 rows, first form with even shares only: 82 -> 58,
 // 57 -> 50, 197 -> 148, 138 -> 91.  The main loop runs at 1.14k clocks per step of
-// 256 x 256 x 64 (hi and lo: 2 x 8.4 MFLOP a CTA) or at 7 TB/s of weights; what
+// 256 x 256 x 64 (hi and lo: 2 x 8.4 MFLOP a pair) or at 7 TB/s of weights; what
 // is left is each launch's start and its tail (partials, arrival, shares).
 #include "gemm_core.cuh"
 
@@ -94,7 +94,7 @@ __device__ __forceinline__ void load_acc(uint32_t taddr, int lo, float (&v)[kEpi
 // out of its word.  The last contributor to arrive sees, after its own bit, all
 // bits set before that; who gives up later sees the tile complete.  Both calls
 // are rare and out of line: inlined, they lengthened every launch's tail (a
-// batch-16 draft pass: 1640 us, 1599 so; 1588 without giving up at all).
+// batch-16 draft pass: 1640 us, 1599 so; 1545 before shares were given up).
 static __device__ __noinline__ uint32_t claim_shares(unsigned long long* word, uint32_t given) {
   return (uint32_t)(atom_and64(word, ~((unsigned long long)given << kWideContrib)) >> kWideContrib) & given;
 }

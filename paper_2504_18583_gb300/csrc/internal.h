@@ -271,11 +271,12 @@ __host__ __device__ inline void wide_tiles(int m, int& tiles, int& n_tok) {
 // verify of 8 layers, 512-row prompt; us): always even 1673 / 1497 / 18007,
 // with equal parts 1643 / 1426 / 17422, with whole tiles too 1549 / 1384 / 16785
 // at (40, 8); 1566 / 1444 / 16999 at (12, 4), 1562 / 1387 / 16899 at (64, 8).
-// Fewer tiles than pairs stay whole only up to kWideWhole units: the tensor
-// cores truncate at every accumulation (hi and lo parts: eight a unit), and
-// with the QKV projection's 64 units in one accumulator the keys' and values'
-// bf16 roundings moved the error of 6 layers over a 512-row prompt from
-// 1.36e-3 to 1.57e-3 (1.38e-3 with the even split, at the same speed).
+// Fewer tiles than pairs, and more than half as many, stay whole up to
+// kWideWhole units, as the 1B draft's gate/up does; the even split makes its
+// passes of more than 64 rows 5% to 8% slower.  With the limit above 64 units
+// the QKV projection of the 8B widths would sum two pieces of kWideChain units
+// a tile instead of even shares of 20: 1% to 2% off a 512-row prompt, but its
+// error, and a batch-16 verify pass's, 3% to 4% larger.
 constexpr int kWideExchange = 40, kWideSecond = 8, kWideWhole = 32;
 struct WideSplit {
   int pairs;
@@ -321,7 +322,7 @@ constexpr int kCodMaxN = 4096;  // rows per subtask of one COD sample
 void launch_cod(int N, int K, double r, double r_min, uint64_t seed, uint64_t sample_id, int32_t* keep,
                 int32_t* counts, cudaStream_t s);
 void launch_gemm(const GemmArgs& a, int tt, int grid, cudaStream_t s, bool pdl);
-int gemm_wide_max_pairs(int sm);  // pairs the GPU holds at once (all of a launch's pairs must be)
+int gemm_wide_max_pairs(int sm);  // pairs an idle GPU holds at once: a launch has no more
 void launch_gemm_wide(const WideArgs& a, int pairs, cudaStream_t s, bool pdl);
 void launch_attention(const AttnArgs& a, int grid_x, cudaStream_t s, bool pdl);
 int attention_rows_per_block(int group);

@@ -567,8 +567,12 @@ __global__ void __launch_bounds__(kResampleThreads) resample_kernel(const __grid
   // A thread takes the four entries of one Philox block at a time.  An entry
   // whose noise cannot lift it over the warp's best so far is passed over
   // before the logarithms: its score beats `best` only if -log u < w exp(-best)
-  // (w exp(-best) = exp(y/T - best) without a draft row), and -log u >= 1 - u;
-  // the factor 1.0001 is far above the roundings of both sides.
+  // (w exp(-best) = exp(y/T - best) without a draft row), and -log u >= 1 - u.
+  // The factor 1.0001 is far above the errors of the exponentials and of the
+  // noise (1e-5 together), so the exact sum of an entry passed over is below
+  // `best`; rounded, at whatever size y/T gives it, it is at most `best`, and
+  // an equal score of a later entry does not win: the warp's best is of an
+  // earlier round of the loop, whose indices are all lower.
   const uint64_t seed = a.call.seed;
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32), step = (uint32_t)a.call.step;
   const float cy = nm.x / T, cz = nm.z / T;
@@ -655,8 +659,9 @@ void launch_accept_sample(const AcceptArgs& a, cudaStream_t s, bool pdl) {
 // Tile statistics of given logits rows (same layout as the LM-head
 // epilogue): per 128-entry tile the max and argmax, the sum of exp((x - max)/T)
 // and, when gumbel_stream >= 0 and the call samples, the Gumbel-max winner of
-// the tile for row m = b * rows_per_seq + i (Philox row i of sequence b), the
-// draw the LM-head epilogue makes for a draft row.
+// the tile for row m = b * rows_per_seq + i (Philox row i of sequence b): the
+// draw that the LM-head epilogue makes for a draft row, by scoring every entry
+// exactly (the epilogue ranks roughly first).
 __global__ void __launch_bounds__(128) row_stats_kernel(const float* logits, int vocab, int m_cap, const CallArgs* call,
                                                         int gumbel_stream, int rows_per_seq, float4* stats,
                                                         int2* stats_i) {

@@ -283,7 +283,7 @@ def test_autoregressive_mode_k0_matches_the_oracle_forward():
 def test_batch16_ragged_full_width_two_layers():
     """The batch-16 ragged configuration (8b_batch16: K = 6, ragged prompts)
     at full width with two layers per model: 16 x 7 = 112 verify rows and 192
-    draft rows take the 64-token tiles, and attention covers 16 sequences of
+    draft rows take the CTA pairs' tiles, and attention covers 16 sequences of
     different lengths.  Prompts are 16..64 tokens here (the configuration's
     128..2048 keep the CPU oracle's prefill within seconds only at this size)."""
     wl = S.WORKLOADS["8b_batch16"].replace(target=S.TARGET_8B.replace(n_layers=2),
@@ -403,10 +403,12 @@ def test_vanilla_sd_sampled_sequential_draft():
 @pytest.mark.parametrize("vocab", [2048, 128256])
 def test_draft_sampler_on_identical_logits(vocab):
     """Level 1 for the draft's candidate selection (Eq. 6, sampled at
-    temperature T, and greedy): given draft logits go through the same tile
-    statistics and selection kernel as the LM head's, and the candidates
-    equal the oracle's Gumbel-max (or argmax) winners on the same Philox
-    stream exactly, except where the winner's lead is a few fp32 ulps."""
+    temperature T, and greedy): given draft logits go through statistics of
+    the LM head's layout, every entry scored exactly, and the same selection
+    kernel, and the candidates equal the oracle's Gumbel-max (or argmax)
+    winners on the same Philox stream exactly, except where the winner's lead
+    is a few fp32 ulps.  (The LM head's own draw:
+    test_lm_head_draw_follows_its_own_logits.)"""
     import torch
     wl = S.WORKLOADS["tiny"].replace(batch=3, K=6, n_new=100, prompt_len=20)
     if vocab != wl.target.vocab:
