@@ -71,7 +71,7 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], uint32_t addr) {
 // Against expf on natural scores the passes' errors to 64 bits were 0.9993
 // +- 0.0006 times as large (16 cases, 8 seeds each; probabilities are rounded
 // to fp16 next); a batch-16 or prompt pass is 1% to 3% faster so (batch-16
-// draft 1626 us against 1691, 512-row prompt 17.4 ms against 17.8).
+// draft 1624 us against 1691, 512-row prompt 17.3 ms against 17.8).
 __device__ __forceinline__ float exp2_fast(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

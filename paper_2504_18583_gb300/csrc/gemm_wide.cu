@@ -34,11 +34,11 @@
 //
 // Measured (one layer's launches, serialised, us; before: 64-token tiles, and a
 // 128-token tile for gate/up and LM head, on single CTAs): 8B widths, 112 rows:
-// QKV 36 -> 24, O 30 -> 23, gate/up 62 -> 52 (34 at the HBM rate), down 52 -> 36,
-// LM head 236 -> 183; 512 rows, first form with even shares only: 82 -> 58,
-// 57 -> 50, 197 -> 148, 138 -> 91.  The main loop runs at 1.14k clocks per step of
-// 256 x 256 x 64 (hi and lo: 2 x 8.4 MFLOP a pair) or at 7 TB/s of weights; what
-// is left is each launch's start and its tail (partials, arrival, shares).
+// QKV 36 -> 25, O 30 -> 24, gate/up 62 -> 54 (34 at the HBM rate), down 52 -> 38,
+// LM head 236 -> 183; 512 rows: 82 -> 72, 57 -> 44, 197 -> 137, 138 -> 97.
+// The main loop runs at 1.14k clocks per step of 256 x 256 x 64 (hi and lo: 2 x
+// 8.4 MFLOP a pair) or at 7 TB/s of weights; what is left is each launch's start
+// and its tail (partials, arrival, shares).
 #include "gemm_core.cuh"
 
 namespace pard {
